@@ -209,6 +209,12 @@ struct DenseWork {
     bool attr_set = false;
 };
 
+// Workspace of the FP64 tensor-core GEMM (fs_oz.cu): digit images of the projector table
+// (kept), per-call images, row maxima and split-K partial sums.
+struct OzWork {
+    dbuf table_g, table_n, max_g, max_n, aimg, bimg, ma, mb, part;
+};
+
 struct SolverSmall {
     dbuf GA, GB, T1, T2, evals, work, info, theta, act, resid, dots, nrm, shift, dscale, bkin, hres, keep;
     int lwork = 0;
@@ -305,6 +311,7 @@ struct fs_ctx {
     Prof prof;
     Mlp mlp;
     DenseWork dense;
+    OzWork oz;
     SolverMem smem;
     dbuf errflag;     // int: set by a device-side wait that gave up
     int gemm_path = 0;
@@ -394,6 +401,25 @@ void mlp_features(fs_ctx* c, const T2* R, const int* act, int na, const double2*
                   float* zt, float* wt);
 template <typename T2> void mlp_make_w(fs_ctx* c, const T2* R, const int* act, int na, T2* W, const double2* dots);
 template <typename T2> void mlp_err_from_proj(fs_ctx* c, const T2* proj, const T2* X, const int* act, int na, T2* E);
+
+// FP64 GEMM on the tensor cores (fs_oz.cu): operand element (row r, k) at
+// X[map(r) sr + kmap(k) sk] (maps may be null), conjugated where conj; result element
+// (m, n) at C[mmap(m) cm + nmap(n) cn].  table: 1 / 2 when A is the context's projector
+// table with projectors / plane waves as rows (its image is kept).
+struct OzMat {
+    const double2* X;
+    long sr, sk;
+    int conj;
+    const int *map = nullptr, *kmap = nullptr;
+};
+struct OzDst {
+    double2* C;
+    long cm, cn;
+    const int *mmap = nullptr, *nmap = nullptr;
+};
+bool oz_worth(int M, int N, int K);
+void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& A, const OzMat& B, const OzDst& C, double alpha, double beta,
+             int table = 0);
 
 // dense FP64 linear algebra (fs_dense.cu); column-major complex, op 0 = N, 1 = C
 void dense_gemm(fs_ctx* c, int opA, int opB, int M, int N, int K, double alpha, const double2* A, int lda,

@@ -765,6 +765,15 @@ void dense_gemm_impl(fs_ctx* c, int opA, int opB, int M, int N, int K, double al
                      const double2* B, int ldb, double beta, double2* C, int ldc, int lower) {
     if (M <= 0 || N <= 0) return;
     K = std::max(K, 0);
+    // from 6e7 flops on (and 64 k: the digit sums come out once per 64 k) the tensor cores: the FMA
+    // GEMM takes 90 us and more there (0.65 TFLOP/s at best), the digit form 60 to 90 us, all its
+    // passes included, and from 1e9 flops on a tenth
+    if (!lower && oz_worth(M, N, K)) {
+        const OzMat a{A, opA == 0 ? 1l : (long)lda, opA == 0 ? (long)lda : 1l, opA == 1};
+        const OzMat b{B, opB == 0 ? (long)ldb : 1l, opB == 0 ? 1l : (long)ldb, opB == 1};
+        oz_gemm(c, M, N, K, a, b, OzDst{C, 1, ldc}, alpha, beta);
+        return;
+    }
     const int tiles = cdiv(M, TB) * cdiv(N, TB);
     int splits = 1;
     if (tiles < 152 && K >= 8 * TK) splits = std::min(std::max(1, 304 / tiles), std::max(1, K / (4 * TK)));
