@@ -117,11 +117,11 @@ __device__ __forceinline__ uint64_t oz_desc(uint32_t saddr) {
     return d;
 }
 
-// exponent E of a row from the bits of its largest magnitude: |x| < 2^E (127/128 + 2^-8 / 2),
-// the largest number that seven signed digits hold; a mantissa at the top of its range takes
-// the next exponent
+// exponent E of a row from the bits of its largest magnitude.  Seven signed digits hold up to
+// 0x7F7F7F7F7F7F7F = 0.49803 2^56, i.e. |x| <= 0.99607 2^E: a mantissa at the top of its range
+// (six leading ones, |x| >= 0.992 of the next power) takes the next exponent
 __device__ __forceinline__ int oz_exp(unsigned long long bits) {
-    const int e = (int)(bits >> 52) - 1022 + (((bits >> 45) & 0x7f) == 0x7f ? 1 : 0);
+    const int e = (int)(bits >> 52) - 1022 + (((bits >> 46) & 0x3f) == 0x3f ? 1 : 0);
     return e < E_MIN ? E_MIN : e;
 }
 

@@ -61,3 +61,22 @@ def test_scales_and_non_finite_rows(fs):
         keep = [i for i in range(16) if i not in (3, 5, 7)]
         assert np.array_equal(d[keep], a[keep])
         assert not np.isfinite(d[3]).any() and not np.isfinite(d[5]).any() and not d[7].any()
+
+
+def test_row_maxima_at_the_top_of_the_digit_range(fs):
+    # the largest component of a row around 127.5 / 128 of a power of two, where seven signed
+    # digits end (0x7F7F7F7F7F7F7F = 0.996078 2^55) and the next exponent is taken
+    w = fi.make_box(L=(13.0, 13.0, 17.0), n=(24, 24, 32), ecut=6.0, natom=33, widths=(1.0,), lattice=4.0,
+                    nstates=4, e_ref=0.2, seed=23)
+    top = [0.992, 0.9921875, 0.99606, 0.996078, 0.9960784, 0.996080, 0.99609, 0.99609375, 0.9961, 1 - 2.0 ** -53,
+           -0.99608, -(1 - 2.0 ** -53)]
+    with fs.Context.from_workload(w) as c:
+        psi = _psi(len(top), c.npw)
+        psi /= np.maximum(np.abs(psi.real), np.abs(psi.imag)).max(axis=1)[:, None] * 1.1
+        for i, t in enumerate(top):
+            psi[i, 11 * i] = t + 0.25j if i % 2 else 0.25 + 1j * t
+        out = c.apply_H(torch.as_tensor(psi, device="cuda")).cpu().numpy()
+        ref = pw.Hamiltonian(w).apply(psi)
+        tol = 4 * (np.sqrt(c.npw) + 8 * np.log2(24 * 24 * 32)) * 2.0 ** -53
+        for i in range(len(top)):
+            assert rel_err(out[i], ref[i]) < tol, top[i]
