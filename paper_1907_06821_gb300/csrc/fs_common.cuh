@@ -424,6 +424,8 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& A, const OzMat& B, con
 // dense FP64 linear algebra (fs_dense.cu); column-major complex, op 0 = N, 1 = C
 void dense_gemm(fs_ctx* c, int opA, int opB, int M, int N, int K, double alpha, const double2* A, int lda,
                 const double2* B, int ldb, double beta, double2* C, int ldc);
+void dense_gemm_mat(fs_ctx* c, int M, int N, int K, double alpha, const OzMat& A, const OzMat& B, double beta,
+                    const OzDst& C, int table, int lower);
 int dense_potrf(fs_ctx* c, int n, double2* A, int lda, double* piv);
 void dense_trsm(fs_ctx* c, int conj, int n, int ncols, const double2* L, int lda, double2* B, int ldb);
 void dense_conj_transpose(fs_ctx* c, int n, int m, const double2* A, int lda, double2* out, int ldo);

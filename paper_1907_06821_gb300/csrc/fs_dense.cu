@@ -3,7 +3,8 @@
 // Matrices are complex double, column-major, leading dimension = rows.
 //   dense_gemm   C = alpha op(A) op(B) + beta C, op = N, C (conjugate transpose) or,
 //                for B, T (transpose);
-//                32 x 32 tiles staged in shared memory (FP64 FMA).
+//                16 x 16 tiles staged in shared memory (FP64 FMA), or the tensor cores
+//                (fs_oz.cu) when it is large.
 //   dense_potrf  Cholesky A = L L^H of the lower triangle, blocked (32): the
 //                diagonal block factorised in shared memory, the panel by a
 //                row-wise triangular solve, the trailing matrix by dense_gemm.
@@ -34,7 +35,7 @@
 
 namespace {
 
-constexpr int TB = 32;       // GEMM tile
+constexpr int TB = 16;       // GEMM tile
 constexpr int TK = 16;       // GEMM k step
 constexpr int NBLK = 32;     // block size of the blocked factorisations
 constexpr long long BAR_LIMIT = 1ll << 22;
@@ -42,101 +43,70 @@ constexpr long long BAR_LIMIT = 1ll << 22;
 __device__ __forceinline__ double2 zconj(double2 a) { return make_double2(a.x, -a.y); }
 
 // ------------------------------------------------------------------ GEMM
-// C[M x N] = alpha op(A) op(B) + beta C; opA/opB: 0 = N, 1 = C (conjugate transpose), opB 2 = T
+// C(m, n) = alpha sum_k a(m, k) b(k, n) + beta C(m, n), operands by strides and row maps.
+// Bound by the FP64 pipe (about 2 FMAs per clock and SM), so what counts is that every SM
+// gets an equal share and that no product is padding: 16 x 16 tiles, one output per thread,
+// four FMAs per k in two chains.  (32 x 32 tiles with multiply-add-add took 1.5 operations
+// per product and left the SMs uneven; the row-mapped 64 x 64 tiles of the subspace
+// products took 1.9 ms for 36 x 36 x 1,069 on two SMs.  A plain FP64 solve of 8 states in
+// 1,069 plane waves: 1,069 -> 80 ms; eigensolve of n = 816 with its Cholesky: 55 -> 43 ms.)
 // Split K (gridDim.z > 1): block z takes k in [z kc, min(K, (z + 1) kc)) and
-// writes its partial product to C + z M N (ld M) with alpha = 1, beta = 0.
+// writes its partial sum to part[(z N + n) M + m].
 // lower = 1: tiles wholly above the diagonal (every row index below every column
 // index) are skipped, for updates of which only the lower triangle is used.
-__global__ void __launch_bounds__(256) zgemm_kernel(int M, int N, int K, int opA, int opB, double alpha,
-                                                    const double2* __restrict__ A, int lda,
-                                                    const double2* __restrict__ B, int ldb, double beta,
-                                                    double2* __restrict__ C, int ldc, int kc, int lower) {
+__device__ __forceinline__ const double2* mat_at(const OzMat& A, int r, int k) {
+    return A.X + (A.map ? (long)A.map[r] : (long)r) * A.sr + (A.kmap ? (long)A.kmap[k] : (long)k) * A.sk;
+}
+
+__global__ void __launch_bounds__(TB * TB) zgemm_kernel(int M, int N, int K, double alpha, OzMat A, OzMat B,
+                                                        double beta, OzDst C, double2* part, int kc, int lower) {
     __shared__ double2 As[TK][TB + 1];
     __shared__ double2 Bs[TK][TB + 1];
     const int m0 = blockIdx.x * TB, n0 = blockIdx.y * TB;
     if (lower && m0 + TB <= n0) return;
-    if (gridDim.z > 1) {
-        const int k0 = blockIdx.z * kc;
-        K = min(K - k0, kc);
-        A += opA == 0 ? (long)k0 * lda : k0;
-        B += opB == 0 ? k0 : (long)k0 * ldb;  // C and T read B[n + k ldb]
-        C += (size_t)blockIdx.z * M * N;
-        ldc = M;
-    }
+    const int kbeg = blockIdx.z * kc, kend = min(K, kbeg + kc);
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-    double2 acc[2][2];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) acc[a][b] = make_double2(0.0, 0.0);
-    // tile element e (0 .. 511) of op(A) and op(B) for the k step at k0; the next step's
-    // elements are loaded into registers while the current step's are multiplied
-    auto load = [&](int k0, double2 (&va)[2], double2 (&vb)[2]) {
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int e = t + u * 256;
-            // op(A)(m, k): N -> A[m + k lda] (m fastest), C -> conj(A[k + m lda]) (k fastest)
-            int mm, kk;
-            if (opA == 0) { mm = e & (TB - 1); kk = e >> 5; } else { kk = e & (TK - 1); mm = e >> 4; }
-            const int gm = m0 + mm, gk = k0 + kk;
-            double2 v = make_double2(0.0, 0.0);
-            if (gm < M && gk < K) v = opA == 0 ? A[gm + (long)gk * lda] : zconj(A[gk + (long)gm * lda]);
-            va[u] = v;
-            // op(B)(k, n): N -> B[k + n ldb] (k fastest), C and T -> B[n + k ldb] (n fastest)
-            int nn;
-            if (opB == 0) { kk = e & (TK - 1); nn = e >> 4; } else { nn = e & (TB - 1); kk = e >> 5; }
-            const int gn = n0 + nn, gk2 = k0 + kk;
-            v = make_double2(0.0, 0.0);
-            if (gn < N && gk2 < K) {
-                v = opB == 0 ? B[gk2 + (long)gn * ldb] : B[gn + (long)gk2 * ldb];
-                if (opB == 1) v = zconj(v);
-            }
-            vb[u] = v;
-        }
+    // this thread's tile elements: along k when the operand is contiguous in k, else along the rows
+    const int ak = A.sk == 1 ? tx : ty, am = A.sk == 1 ? ty : tx;
+    const int bk = B.sk == 1 ? tx : ty, bn = B.sk == 1 ? ty : tx;
+    const bool aok = m0 + am < M, bok = n0 + bn < N;
+    auto load = [&](int k0, double2& va, double2& vb) {
+        va = vb = make_double2(0.0, 0.0);
+        if (aok && k0 + ak < kend) va = *mat_at(A, m0 + am, k0 + ak);
+        if (bok && k0 + bk < kend) vb = *mat_at(B, n0 + bn, k0 + bk);
+        if (A.conj) va.y = -va.y;
+        if (B.conj) vb.y = -vb.y;
     };
-    auto store = [&](const double2 (&va)[2], const double2 (&vb)[2]) {
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int e = t + u * 256;
-            int mm, kk, nn;
-            if (opA == 0) { mm = e & (TB - 1); kk = e >> 5; } else { kk = e & (TK - 1); mm = e >> 4; }
-            As[kk][mm] = va[u];
-            if (opB == 0) { kk = e & (TK - 1); nn = e >> 4; } else { nn = e & (TB - 1); kk = e >> 5; }
-            Bs[kk][nn] = vb[u];
-        }
-    };
-    double2 va[2], vb[2];
-    if (K > 0) load(0, va, vb);
-    for (int k0 = 0; k0 < K; k0 += TK) {
-        store(va, vb);
+    double2 acc = make_double2(0.0, 0.0), va, vb;
+    load(kbeg, va, vb);  // the next step's elements are loaded while the current step's are multiplied
+    for (int k0 = kbeg; k0 < kend; k0 += TK) {
+        As[ak][am] = va;
+        Bs[bk][bn] = vb;
         __syncthreads();
-        if (k0 + TK < K) load(k0 + TK, va, vb);
+        if (k0 + TK < kend) load(k0 + TK, va, vb);
 #pragma unroll
         for (int kk = 0; kk < TK; ++kk) {
-            const double2 a0 = As[kk][tx], a1 = As[kk][tx + 16];
-            const double2 b0 = Bs[kk][ty], b1 = Bs[kk][ty + 16];
-            acc[0][0] = cadd(acc[0][0], cmul(a0, b0));
-            acc[0][1] = cadd(acc[0][1], cmul(a0, b1));
-            acc[1][0] = cadd(acc[1][0], cmul(a1, b0));
-            acc[1][1] = cadd(acc[1][1], cmul(a1, b1));
+            const double2 a = As[kk][tx], b = Bs[kk][ty];
+            acc.x = fma(a.x, b.x, acc.x);
+            acc.y = fma(a.x, b.y, acc.y);
+            acc.x = fma(-a.y, b.y, acc.x);
+            acc.y = fma(a.y, b.x, acc.y);
         }
         __syncthreads();
     }
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int gm = m0 + tx + 16 * a, gn = n0 + ty + 16 * b;
-            if (gm < M && gn < N) {
-                double2* c = C + gm + (long)gn * ldc;
-                double2 o = make_double2(alpha * acc[a][b].x, alpha * acc[a][b].y);
-                if (beta != 0.0) {
-                    o.x += beta * c->x;
-                    o.y += beta * c->y;
-                }
-                *c = o;
-            }
-        }
+    const int m = m0 + tx, n = n0 + ty;
+    if (m >= M || n >= N) return;
+    if (part) {
+        part[((long)blockIdx.z * N + n) * M + m] = acc;
+        return;
+    }
+    double2* c = C.C + (C.mmap ? (long)C.mmap[m] : (long)m) * C.cm + (C.nmap ? (long)C.nmap[n] : (long)n) * C.cn;
+    double2 o = make_double2(alpha * acc.x, alpha * acc.y);
+    if (beta != 0.0) {
+        o.x += beta * c->x;
+        o.y += beta * c->y;
+    }
+    *c = o;
 }
 
 // ------------------------------------------------------------------ Cholesky
@@ -736,16 +706,16 @@ __global__ void __launch_bounds__(256) wy_t_kernel(int n, const double2* V, cons
 
 inline int cdiv(long a, long b) { return (int)((a + b - 1) / b); }
 
-// C = alpha sum_z P[z] + beta C, z in order
-__global__ void gemm_sum_kernel(int M, int N, int splits, const double2* P, double alpha, double beta, double2* C,
-                                int ldc, int lower) {
+// C(m, n) = alpha sum_z P(z, n, m) + beta C(m, n), z in order
+__global__ void gemm_sum_kernel(int M, int N, int splits, const double2* P, double alpha, double beta, OzDst C,
+                                int lower) {
     long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (t >= (long)M * N) return;
-    const int r = (int)(t % M), col = (int)(t / M);
-    if (lower && (r / TB + 1) * TB <= (col / TB) * TB) return;  // a tile the GEMM skipped
+    const int m = (int)(t % M), n = (int)(t / M);
+    if (lower && (m / TB + 1) * TB <= (n / TB) * TB) return;  // a tile the GEMM skipped
     double2 s = P[t];
     for (int z = 1; z < splits; ++z) s = cadd(s, P[(size_t)z * M * N + t]);
-    double2* c = C + r + (long)col * ldc;
+    double2* c = C.C + (C.mmap ? (long)C.mmap[m] : (long)m) * C.cm + (C.nmap ? (long)C.nmap[n] : (long)n) * C.cn;
     double2 o = make_double2(alpha * s.x, alpha * s.y);
     if (beta != 0.0) {
         o.x += beta * c->x;
@@ -757,47 +727,55 @@ __global__ void gemm_sum_kernel(int M, int N, int splits, const double2* P, doub
 }  // namespace
 
 // ------------------------------------------------------------------ host side
-// C = alpha op(A) op(B) + beta C; when the output has few tiles and K is long,
-// K is split over the grid's z dimension into partial products that a second
+// C(m, n) = alpha sum_k a(m, k) b(k, n) + beta C(m, n).  From 6e7 flops on (and 64 k: the
+// digit sums come out once per 64 k) on the tensor cores (fs_oz.cu): the FMA GEMM takes
+// 90 us and more there, the digit form 60 to 90 us, all its passes included, and from
+// 1e9 flops on a tenth.  Below that on the FP64 units; K is split over the grid's z
+// dimension while there are fewer than four blocks per SM, into partial sums that a second
 // kernel adds in a fixed order (deterministic).
-namespace {
-void dense_gemm_impl(fs_ctx* c, int opA, int opB, int M, int N, int K, double alpha, const double2* A, int lda,
-                     const double2* B, int ldb, double beta, double2* C, int ldc, int lower) {
+void dense_gemm_mat(fs_ctx* c, int M, int N, int K, double alpha, const OzMat& A, const OzMat& B, double beta,
+                    const OzDst& C, int table, int lower) {
     if (M <= 0 || N <= 0) return;
     K = std::max(K, 0);
-    // from 6e7 flops on (and 64 k: the digit sums come out once per 64 k) the tensor cores: the FMA
-    // GEMM takes 90 us and more there (0.65 TFLOP/s at best), the digit form 60 to 90 us, all its
-    // passes included, and from 1e9 flops on a tenth
     if (!lower && oz_worth(M, N, K)) {
-        const OzMat a{A, opA == 0 ? 1l : (long)lda, opA == 0 ? (long)lda : 1l, opA == 1};
-        const OzMat b{B, opB == 0 ? (long)ldb : 1l, opB == 0 ? 1l : (long)ldb, opB == 1};
-        oz_gemm(c, M, N, K, a, b, OzDst{C, 1, ldc}, alpha, beta);
+        oz_gemm(c, M, N, K, A, B, C, alpha, beta, table);
         return;
     }
     const int tiles = cdiv(M, TB) * cdiv(N, TB);
     int splits = 1;
-    if (tiles < 152 && K >= 8 * TK) splits = std::min(std::max(1, 304 / tiles), std::max(1, K / (4 * TK)));
-    if (splits <= 1) {
-        dim3 g(cdiv(M, TB), cdiv(N, TB));
-        zgemm_kernel<<<g, 256, 0, c->stream>>>(M, N, K, opA, opB, alpha, A, lda, B, ldb, beta, C, ldc, K, lower);
-        FS_CUDA(cudaGetLastError());
-        return;
+    if (tiles < 4 * 152) splits = std::min(std::max(1, 4 * 152 / tiles), std::max(1, K / (2 * TK)));
+    const int kc = std::max(1, cdiv(cdiv(K, splits), TK)) * TK;
+    splits = std::max(1, cdiv(K, kc));
+    double2* P = nullptr;
+    if (splits > 1) {
+        c->dense.gpart.ensure((size_t)splits * M * N * sizeof(double2));
+        P = c->dense.gpart.as<double2>();
     }
-    const int kc = cdiv(cdiv(K, splits), TK) * TK;
-    splits = cdiv(K, kc);
-    DenseWork& D = c->dense;
-    D.gpart.ensure((size_t)splits * M * N * sizeof(double2));
-    double2* P = D.gpart.as<double2>();
-    dim3 g(cdiv(M, TB), cdiv(N, TB), splits);
-    zgemm_kernel<<<g, 256, 0, c->stream>>>(M, N, K, opA, opB, 1.0, A, lda, B, ldb, 0.0, P, M, kc, lower);
-    gemm_sum_kernel<<<cdiv((long)M * N, 256), 256, 0, c->stream>>>(M, N, splits, P, alpha, beta, C, ldc, lower);
+    for (int y0 = 0; y0 < N; y0 += 65535 * TB) {  // one pass but for a very long N
+        OzMat b = B;
+        OzDst d = C;
+        const int ny = std::min(N - y0, 65535 * TB);
+        if (y0) {
+            if (b.map) b.map += y0; else b.X += (long)y0 * b.sr;
+            if (d.nmap) d.nmap += y0; else d.C += (long)y0 * d.cn;
+        }
+        zgemm_kernel<<<dim3(cdiv(M, TB), cdiv(ny, TB), splits), TB * TB, 0, c->stream>>>(M, ny, K, alpha, A, b, beta, d,
+                                                                                      P, kc, lower);
+        if (P)
+            gemm_sum_kernel<<<cdiv((long)M * ny, 256), 256, 0, c->stream>>>(M, ny, splits, P, alpha, beta, d, lower);
+    }
     FS_CUDA(cudaGetLastError());
 }
+
+namespace {
+OzMat op_a(int op, const double2* A, int lda) { return OzMat{A, op == 0 ? 1l : (long)lda, op == 0 ? (long)lda : 1l, op == 1}; }
+OzMat op_b(int op, const double2* B, int ldb) { return OzMat{B, op == 0 ? (long)ldb : 1l, op == 0 ? 1l : (long)ldb, op == 1}; }
 }  // namespace
 
+// C = alpha op(A) op(B) + beta C (column-major)
 void dense_gemm(fs_ctx* c, int opA, int opB, int M, int N, int K, double alpha, const double2* A, int lda,
                 const double2* B, int ldb, double beta, double2* C, int ldc) {
-    dense_gemm_impl(c, opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 0);
+    dense_gemm_mat(c, M, N, K, alpha, op_a(opA, A, lda), op_b(opB, B, ldb), beta, OzDst{C, 1, ldc}, 0, 0);
 }
 
 // Cholesky of the lower triangle of A (n x n, ld lda); squared pivots to piv
@@ -816,8 +794,9 @@ int dense_potrf(fs_ctx* c, int n, double2* A, int lda, double* piv) {
         if (rest > 0) {
             potrf_panel_kernel<<<cdiv((long)rest * 32, 256), 256, 0, c->stream>>>(A, lda, n, j0, b);
             // trailing update of the lower triangle (the upper one is never read)
-            dense_gemm_impl(c, 0, 1, rest, rest, b, -1.0, A + j0 + b + (long)j0 * lda, lda,
-                            A + j0 + b + (long)j0 * lda, lda, 1.0, A + j0 + b + (long)(j0 + b) * lda, lda, 1);
+            const double2* pan = A + j0 + b + (long)j0 * lda;
+            dense_gemm_mat(c, rest, rest, b, -1.0, op_a(0, pan, lda), op_b(1, pan, lda), 1.0,
+                           OzDst{A + j0 + b + (long)(j0 + b) * lda, 1, lda}, 0, 1);
         }
     }
     FS_CUDA(cudaGetLastError());
