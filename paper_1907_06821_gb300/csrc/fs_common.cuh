@@ -205,7 +205,7 @@ constexpr size_t FS_FMT_CHUNK_BYTES = 4ull << 30;
 // Workspace of the dense FP64 linear algebra (fs_dense.cu), kept by the context.
 #define FS_DENSE_MAX_N 2048
 struct DenseWork {
-    dbuf V, tau, d, e, e2, Y, z, work, info3, bar, info, T, U, wyG, wyT, wyW, wyW2, gpart, qrG, qrT;
+    dbuf V, tau, d, e, e2, Y, z, work, info3, info, T, U, wyG, wyT, wyW, wyW2, gpart, qrG, qrT, linv, xb, ds;
     bool attr_set = false;
 };
 
@@ -394,6 +394,7 @@ int mlp_nparam();
 void mlp_setup(fs_ctx* c);
 void mlp_prepare(fs_ctx* c);
 void mlp_forward(fs_ctx* c, const float* F, int rows, float* z);
+double mlp_weight_sum(fs_ctx* c, const float* wt, int rows);
 double mlp_loss_grad(fs_ctx* c, const float* F, const float* zt, const float* wt, int rows, double sw);
 void mlp_adam(fs_ctx* c, float lr);
 template <typename T2>
@@ -427,7 +428,8 @@ void dense_gemm(fs_ctx* c, int opA, int opB, int M, int N, int K, double alpha, 
 void dense_gemm_mat(fs_ctx* c, int M, int N, int K, double alpha, const OzMat& A, const OzMat& B, double beta,
                     const OzDst& C, int table, int lower);
 int dense_potrf(fs_ctx* c, int n, double2* A, int lda, double* piv);
-void dense_trsm(fs_ctx* c, int conj, int n, int ncols, const double2* L, int lda, double2* B, int ldb);
+void dense_trsm(fs_ctx* c, int conj, int n, int ncols, const double2* L, int lda, double2* B, int ldb,
+                bool fresh = true);
 void dense_conj_transpose(fs_ctx* c, int n, int m, const double2* A, int lda, double2* out, int ldo);
 void dense_heev(fs_ctx* c, int n, double2* A, int m, double* w, double2* Z, int ldz);
 int dense_hegv(fs_ctx* c, int n, double2* GA, double2* GB, int m, double* w);

@@ -13,8 +13,8 @@
 //   dense_heev   the m lowest eigenpairs of a Hermitian matrix:
 //     1. Householder reduction to a real symmetric tridiagonal T = Q^H A Q
 //        (Q = H_0 ... H_{n-2}, H_i = I - tau_i v_i v_i^H, the LAPACK zhetd2
-//        steps), all n - 1 steps in one cooperative kernel whose blocks meet
-//        at a bounded grid barrier twice per step;
+//        steps), all n - 1 steps in one cooperative kernel whose blocks exchange
+//        one vector per step (bounded waits);
 //     2. eigenvalues of T by bisection on Sturm counts (a warp evaluates 31
 //        points of the bracket at once, so each round narrows it 32-fold; the
 //        counts come from the leading minors, rescaled, without division);
@@ -24,7 +24,7 @@
 //        other by modified Gram-Schmidt (a warp per cluster);
 //     4. back-transformation Z = Q z in blocks of 32 reflectors (compact WY
 //        form), each block as three GEMMs, then one Cholesky QR pass on Z.
-// Every device-side wait (the grid barrier) is bounded: on expiry the
+// Every device-side wait (the exchange of the reduction) is bounded: on expiry the
 // context's error flag is raised and the kernel returns.
 #include "fs_common.cuh"
 
@@ -38,7 +38,8 @@ namespace {
 constexpr int TB = 16;       // GEMM tile
 constexpr int TK = 16;       // GEMM k step
 constexpr int NBLK = 32;     // block size of the blocked factorisations
-constexpr long long BAR_LIMIT = 1ll << 22;
+constexpr long long BAR_LIMIT = 1ll << 22;  // polls of a wait before it gives up
+constexpr int HETRD_SMEM = 224 * 1024;
 
 __device__ __forceinline__ double2 zconj(double2 a) { return make_double2(a.x, -a.y); }
 
@@ -110,32 +111,40 @@ __global__ void __launch_bounds__(TB * TB) zgemm_kernel(int M, int N, int K, dou
 }
 
 // ------------------------------------------------------------------ Cholesky
-// Factor the b x b diagonal block at A + j0 (1 + lda) in shared memory; squared
-// pivots to piv[j0 + j]; the first non-positive pivot sets *info = j0 + j + 1
-// (once) and is replaced by 1 so that the arithmetic stays finite.
-__global__ void potrf_diag_kernel(double2* A, int lda, int j0, int b, double* piv, int* info) {
-    __shared__ double2 S[NBLK][NBLK + 1];
+// Factor the b x b diagonal block at A + j0 (1 + lda); squared pivots to piv[j0 + j]; the
+// first non-positive pivot sets *info = j0 + j + 1 (once) and is replaced by 1 so that the
+// arithmetic stays finite.  Thread (lane r, warp c) keeps element (r, c) in a register; warp j
+// scales column j and hands it over in shared memory, one barrier per column (the chain of a
+// column: reciprocal square root, scaling, barrier, rank-1 term; with the pivot on one thread
+// and three barriers a block took 40 us).
+__global__ void __launch_bounds__(NBLK * NBLK) potrf_diag_kernel(double2* A, int lda, int j0, int b, double* piv,
+                                                                 int* info) {
+    __shared__ double2 col[2][NBLK];
     const int r = threadIdx.x & (NBLK - 1), c = threadIdx.x >> 5;  // 1024 threads
     double2* D = A + j0 + (long)j0 * lda;
-    if (r < b && c < b) S[r][c] = D[r + (long)c * lda];
-    __syncthreads();
+    double2 a = make_double2(0.0, 0.0);
+    if (r < b && c < b && r >= c) a = D[r + (long)c * lda];
     for (int j = 0; j < b; ++j) {
-        if (threadIdx.x == 0) {
-            double p = S[j][j].x;
-            if (piv) piv[j0 + j] = p;
-            if (!(p > 0.0)) {
-                atomicCAS(info, 0, j0 + j + 1);
-                p = 1.0;
+        if (c == j) {
+            double p = __shfl_sync(0xffffffffu, a.x, j);
+            const bool bad = !(p > 0.0);
+            if (r == j) {
+                if (piv) piv[j0 + j] = p;
+                if (bad) atomicCAS(info, 0, j0 + j + 1);
             }
-            S[j][j] = make_double2(sqrt(p), 0.0);
+            if (bad) p = 1.0;
+            const double inv = rsqrt(p);
+            a = r == j ? make_double2(p * inv, 0.0) : cscale(a, inv);
+            col[j & 1][r] = a;
         }
         __syncthreads();
-        if (c == j && r > j && r < b) S[r][j] = cscale(S[r][j], 1.0 / S[j][j].x);
-        __syncthreads();
-        if (c > j && r >= c && r < b) S[r][c] = csub(S[r][c], cmul(S[r][j], zconj(S[c][j])));
-        __syncthreads();
+        if (c > j && r >= c) {
+            const double2 x = col[j & 1][r], y = col[j & 1][c];  // a -= x conj(y)
+            a.x = fma(-x.x, y.x, fma(-x.y, y.y, a.x));
+            a.y = fma(x.x, y.y, fma(-x.y, y.x, a.y));
+        }
     }
-    if (r < b && c < b && r >= c) D[r + (long)c * lda] = S[r][c];
+    if (r < b && c < b && r >= c) D[r + (long)c * lda] = a;
 }
 
 // rows r >= j0 + b of the panel: A[r, j0:j0+b] <- A[r, j0:j0+b] L^-H (L the
@@ -144,7 +153,8 @@ __global__ void potrf_panel_kernel(double2* A, int lda, int n, int j0, int b) {
     __shared__ double2 Ls[NBLK][NBLK + 1];
     for (int i = threadIdx.x; i < b * b; i += blockDim.x) {
         const int rr = i % b, cc = i / b;
-        Ls[rr][cc] = A[j0 + rr + (long)(j0 + cc) * lda];
+        const double2 l = A[j0 + rr + (long)(j0 + cc) * lda];
+        Ls[rr][cc] = rr == cc ? make_double2(1.0 / l.x, 0.0) : l;  // reciprocals on the diagonal
     }
     __syncthreads();
     const int lane = threadIdx.x & 31;
@@ -153,42 +163,68 @@ __global__ void potrf_panel_kernel(double2* A, int lda, int n, int j0, int b) {
     double2 xv = lane < b ? A[r + (long)(j0 + lane) * lda] : make_double2(0.0, 0.0);
     // x_c = (a_c - sum_{k<c} x_k conj(L[c][k])) / L[c][c]
     for (int c = 0; c < b; ++c) {
-        if (lane == c) xv = cscale(xv, 1.0 / Ls[c][c].x);
+        if (lane == c) xv = cscale(xv, Ls[c][c].x);
         const double2 xc = make_double2(__shfl_sync(0xffffffffu, xv.x, c), __shfl_sync(0xffffffffu, xv.y, c));
-        if (lane > c && lane < b) xv = csub(xv, cmul(xc, zconj(Ls[lane][c])));
+        if (lane > c && lane < b) {
+            const double2 l = Ls[lane][c];
+            xv.x = fma(-xc.x, l.x, fma(-xc.y, l.y, xv.x));
+            xv.y = fma(xc.x, l.y, fma(-xc.y, l.x, xv.y));
+        }
     }
     if (lane < b) A[r + (long)(j0 + lane) * lda] = xv;
 }
 
 // ------------------------------------------------------------------ triangular solves
-// Diagonal block solve for every column: conj = 0: x = L_bb^-1 b (forward);
-// conj = 1: x = L_bb^-H b (backward).  One warp per column, lane r holding row r.
-__global__ void trsm_diag_kernel(const double2* L, int lda, int j0, int b, double2* B, int ldb, int ncols, int conj) {
-    __shared__ double2 Ls[NBLK][NBLK + 1];
-    for (int i = threadIdx.x; i < b * b; i += blockDim.x) {
-        const int rr = i % b, cc = i / b;
-        Ls[rr][cc] = L[j0 + rr + (long)(j0 + cc) * lda];
+// Inverses of the IB x IB diagonal blocks of the lower triangular L, all in one launch: a
+// warp per column j of a block solves L x = e_j (lane l holding rows l, l + 32, ..).  Block
+// b goes to X + b IB IB (ld IB), zeros above the diagonal.  With them a triangular solve is
+// GEMMs alone, of 128 k a step (on the tensor cores when the right-hand sides are many)
+// instead of 32 with a substitution kernel between: n = 816, 816 columns: 3.3 ms before.
+constexpr int IB = 128;
+__global__ void __launch_bounds__(128) tri_inv_kernel(const double2* L, int lda, int n, double2* X) {
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int j0 = (w / IB) * IB, j = w % IB, b = min(IB, n - j0);
+    if (j0 >= n || j >= b) return;
+    const double2* D = L + j0 + (long)j0 * lda;
+    double2* out = X + (long)j0 * IB + (long)j * IB;
+    double2 x[IB / 32];
+    double id[IB / 32];  // reciprocals of the diagonal entries
+#pragma unroll
+    for (int q = 0; q < IB / 32; ++q) {
+        const int r = lane + 32 * q;
+        x[q] = make_double2(r == j ? 1.0 : 0.0, 0.0);
+        id[q] = r >= j && r < b ? 1.0 / D[r + (long)r * lda].x : 0.0;
     }
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (col >= ncols) return;
-    double2* x = B + j0 + (long)col * ldb;
-    double2 v = lane < b ? x[lane] : make_double2(0.0, 0.0);
-    if (!conj) {
-        for (int r = 0; r < b; ++r) {
-            if (lane == r) v = cscale(v, 1.0 / Ls[r][r].x);
-            const double2 xr = make_double2(__shfl_sync(0xffffffffu, v.x, r), __shfl_sync(0xffffffffu, v.y, r));
-            if (lane > r && lane < b) v = csub(v, cmul(Ls[lane][r], xr));
+    // column k of L, the next one loaded while the current one is used
+    auto load = [&](int k, double2 (&lk)[IB / 32]) {
+#pragma unroll
+        for (int q = 0; q < IB / 32; ++q) {
+            const int r = lane + 32 * q;
+            lk[q] = r > k && r < b ? D[r + (long)k * lda] : make_double2(0.0, 0.0);
         }
-    } else {
-        for (int r = b - 1; r >= 0; --r) {
-            if (lane == r) v = cscale(v, 1.0 / Ls[r][r].x);
-            const double2 xr = make_double2(__shfl_sync(0xffffffffu, v.x, r), __shfl_sync(0xffffffffu, v.y, r));
-            if (lane < r) v = csub(v, cmul(zconj(Ls[r][lane]), xr));
+    };
+    double2 nx[IB / 32];
+    load(j, nx);
+#pragma unroll
+    for (int g = 0; g < IB / 32; ++g) {
+        if (32 * g + 31 < j || 32 * g >= b) continue;
+        for (int l = max(0, j - 32 * g); l < min(32, b - 32 * g); ++l) {
+            const int k = 32 * g + l;
+            double2 lk[IB / 32];
+#pragma unroll
+            for (int q = 0; q < IB / 32; ++q) lk[q] = nx[q];
+            load(k + 1, nx);  // (rows beyond k + 1 only: none for the last column)
+            if (lane == l) x[g] = cscale(x[g], id[g]);
+            const double2 xk = make_double2(__shfl_sync(0xffffffffu, x[g].x, l), __shfl_sync(0xffffffffu, x[g].y, l));
+#pragma unroll
+            for (int q = g; q < IB / 32; ++q) {
+                x[q].x = fma(-lk[q].x, xk.x, fma(lk[q].y, xk.y, x[q].x));
+                x[q].y = fma(-lk[q].x, xk.y, fma(-lk[q].y, xk.x, x[q].y));
+            }
         }
     }
-    if (lane < b) x[lane] = v;
+#pragma unroll
+    for (int q = 0; q < IB / 32; ++q) out[lane + 32 * q] = lane + 32 * q < b ? x[q] : make_double2(0.0, 0.0);
 }
 
 __global__ void conj_transpose_kernel(int n, int m, const double2* A, int lda, double2* out, int ldo) {
@@ -196,6 +232,14 @@ __global__ void conj_transpose_kernel(int n, int m, const double2* A, int lda, d
     if (t >= (long)n * m) return;
     const int r = (int)(t % n), c = (int)(t / n);
     out[c + (long)r * ldo] = zconj(A[r + (long)c * lda]);
+}
+
+// Z (n x m) = T^H (T m x n) unless *info
+__global__ void qr_back_kernel(int n, int m, const double2* T, double2* Z, int ldz, const int* info) {
+    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (t >= (long)n * m || *info) return;
+    const int r = (int)(t % n), c = (int)(t / n);
+    Z[r + (long)c * ldz] = zconj(T[c + (long)r * m]);
 }
 
 // A <- (A + A^H) / 2 (exactly Hermitian input for the reduction)
@@ -211,228 +255,263 @@ __global__ void hermitize_kernel(double2* A, int n) {
     if (r == c) A[r + (long)c * n].y = 0.0;
 }
 
-// ------------------------------------------------------------------ grid barrier
-// Blocks of a cooperative launch meet here.  Bounded: after BAR_LIMIT polls the
-// waiting block raises the error flag and reports failure.
-__device__ bool grid_barrier(unsigned int* bar, unsigned int nblocks, int* err) {
-    __shared__ int ok_s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        ok_s = 1;
-        volatile unsigned int* gen = bar + 1;
-        const unsigned int g = *gen;
-        __threadfence();
-        if (atomicAdd(bar, 1u) == nblocks - 1) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-        } else {
-            long long it = 0;
-            while (*gen == g) {
-                if (++it > BAR_LIMIT || *(volatile int*)err) {
-                    atomicExch(err, 1);
-                    ok_s = 0;
-                    break;
-                }
-                __nanosleep(64);
-            }
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return ok_s != 0;
-}
-
-__device__ double block_sum(double v, double* red) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-    __syncthreads();
-    if (l == 0) red[w] = v;
-    __syncthreads();
-    double s = 0;
-    for (int i = 0; i < nw; ++i) s += red[i];
-    return s;
-}
-
 // ------------------------------------------------------------------ tridiagonal reduction
 // Full Hermitian A (n x n, both triangles).  Step i: reflector v_i (v[0] = 1 at
 // row i + 1) with H^H x = beta e_1 for x = A[i+1:, i]; y_i = A22 v_i;
 // s_i = v_i^H y_i; w_i = tau_i y_i - (|tau_i|^2 s_i / 2) v_i;
 // A22 -= v_i w_i^H + w_i v_i^H.  Outputs: d, e (real), tau, V[:, i] = v_i.
 //
-// One grid barrier per step: after it, every block forms w_i from the segment
-// sums of y_i, rebuilds the updated column i + 1 itself (old column minus the
-// rank-2 term; no block writes that column) and from it the reflector v_{i+1};
-// then (column, segment of SEG rows) units update A22 in place and, from the
-// values they just wrote, form the segment sums of y_{i+1}.  Row i + 1 and
-// column i + 1 of A are never updated in place: they are not read again.
-constexpr int SEG = 256;
+// All n - 1 steps in one cooperative kernel.  Block b owns the columns j = b mod gridDim.x
+// (in shared memory when they fit, else in place) and thread t of every block the rows
+// r = t mod HT, whose parts of v and w it keeps in registers.  In a step a block brings its
+// columns up to date, forms y_i[j] = <column j, v_i> for them and publishes these numbers
+// (and, from the owner of column i + 1, that column); every block then forms w_i, the
+// updated column i + 1 and the next reflector for itself.  The published numbers are their
+// own flags: Y and C have a row per step, filled with a NaN pattern beforehand, and the
+// readers poll until every entry has changed, so a step costs one store and one load
+// through L2 instead of a grid barrier, a segment sum and three reads of A.
+// Bound: FP64 rate (12 operations per element of A22 and step, 20 per row and block) and
+// about 6 us a step of dependent FP64 operations and L2 round trips.  Four warps, one per
+// scheduler: what every warp computes for itself (the reflector's scalars, the sums) then
+// costs its own pipe only; eight took 45 % longer at n = 108.  Measured: n = 816: 20.0 ->
+// 13.5 ms, n = 204: 2.3 -> 1.5 ms.
+constexpr unsigned long long EMPTY = 0xffffffffffffffffull;     // a NaN that no arithmetic returns
 
-// reflector from x[0..L) (smem v holds x on entry, v on exit); every block
-__device__ void make_reflector(double2* v, int L, double* red, double2& tau_out, double& beta_out) {
-    __shared__ double2 sh_tau, sh_sc;
-    __shared__ double sh_beta;
-    double ss = 0;
-    for (int k = 1 + threadIdx.x; k < L; k += blockDim.x) ss += v[k].x * v[k].x + v[k].y * v[k].y;
-    const double xn2 = block_sum(ss, red);
-    if (threadIdx.x == 0) {
-        const double2 al = v[0];
-        if (xn2 == 0.0 && al.y == 0.0) {  // nothing to eliminate: H = I
-            sh_tau = make_double2(0.0, 0.0);
-            sh_beta = al.x;
-            sh_sc = make_double2(0.0, 0.0);
-        } else {
-            const double beta = -copysign(sqrt(al.x * al.x + al.y * al.y + xn2), al.x);
-            sh_tau = make_double2((beta - al.x) / beta, -al.y / beta);
-            sh_beta = beta;
-            const double2 den = make_double2(al.x - beta, al.y);  // 1 / (alpha - beta)
-            const double dd = den.x * den.x + den.y * den.y;
-            sh_sc = make_double2(den.x / dd, -den.y / dd);
-        }
-    }
-    __syncthreads();
-    const double2 sc = sh_sc;
-    for (int k = threadIdx.x; k < L; k += blockDim.x) v[k] = k == 0 ? make_double2(1.0, 0.0) : cmul(v[k], sc);
-    tau_out = sh_tau;
-    beta_out = sh_beta;
-    __syncthreads();
+__device__ __forceinline__ void publish(double* p, double v) {
+    if ((unsigned long long)__double_as_longlong(v) == EMPTY) v = __longlong_as_double(0x7ff8000000000000ll);
+    asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
+}
+__device__ __forceinline__ double2 peek(const double2* p) {
+    double2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ bool is_empty(double2 v) {
+    return (unsigned long long)__double_as_longlong(v.x) == EMPTY || (unsigned long long)__double_as_longlong(v.y) == EMPTY;
 }
 
-__global__ void __launch_bounds__(256)
-hetrd_kernel(int n, double2* A, double2* V, double2* tau, double* d, double* e, double2* Yp, unsigned int* bar,
+// 1 / sqrt(s) and 1 / s for normal s > 0 by Newton's iteration from a single-precision start on
+// the mantissa (an FP64 instruction holds a warp's pipe for 64 cycles, and the library forms
+// take three times as many of them): relative error below 2^-51
+__device__ __forceinline__ double newton_rsqrt(double s) {
+    const int h = __double2hiint(s), ex = ((h >> 20) - 1023) & ~1;  // even part of the exponent
+    const double m = __hiloint2double(h - (ex << 20), __double2loint(s));  // in [1, 4)
+    double y = (double)rsqrtf((float)m);
+    const double hm = 0.5 * m;
+    y = y * fma(-hm * y, y, 1.5);
+    y = fma(y * fma(-hm * y, y, 0.5), 1.0, y);
+    return __hiloint2double(__double2hiint(y) - ((ex / 2) << 20), __double2loint(y));
+}
+__device__ __forceinline__ double newton_rcp(double s) {
+    const int h = __double2hiint(s), ex = (h >> 20) - 1023;
+    const double m = __hiloint2double(h - (ex << 20), __double2loint(s));  // in [1, 2)
+    double y = (double)(1.0f / (float)m);
+    y = fma(y, fma(-m, y, 1.0), y);
+    y = fma(y, fma(-m, y, 1.0), y);
+    return __hiloint2double(__double2hiint(y) - (ex << 20), __double2loint(y));
+}
+
+// sum over the block of one double per thread, given to every thread; red: HT / 32 doubles
+// that no other use touches until the next barrier
+template <int HT> __device__ __forceinline__ double ht_sum(double v, double* red) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = red[threadIdx.x & (HT / 32 - 1)];
+    for (int o = HT / 64; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+template <int HT, int PER>
+__global__ void __launch_bounds__(HT)
+hetrd_kernel(int n, double2* A, double2* V, double2* tau, double* d, double* e, double2* Y, double2* C, int in_smem,
              int* err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2* v = reinterpret_cast<double2*>(smem_raw);  // v_i (length n - i - 1)
-    double2* w = v + n;                                  // w_i
-    double2* vn = w + n;                                 // v_{i+1}
-    __shared__ double red[32];
-    const unsigned int nb = gridDim.x;
-    const int lane = threadIdx.x & 31;
-    const int gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    constexpr int PER = SEG / 32;
+    double2* sv = reinterpret_cast<double2*>(smem_raw);  // v_{i-1} and w_{i-1} by row
+    double2* sw = sv + n;
+    const int nb = gridDim.x, bid = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+    const int nown = (n - bid + nb - 1) / nb;  // owned columns bid, bid + nb, ...
+    double2* cols = in_smem ? sw + n : A + (long)bid * n;
+    const long cstr = in_smem ? n : (long)nb * n;
+    double2* part = in_smem ? sw + n + (long)((n + nb - 1) / nb) * n : sw + n;  // [nown][HT / 32]
+    __shared__ double red[2][HT / 32];
+    __shared__ double2 head[2];  // broadcast of y[i + 1] and of the head of the next reflector
+    __shared__ int gave_up;
+    if (tid == 0) gave_up = 0;
     if (n < 2) {
-        if (blockIdx.x == 0 && threadIdx.x == 0 && n == 1) d[0] = A[0].x;
+        if (bid == 0 && tid == 0 && n == 1) d[0] = A[0].x;
         return;
     }
-    // step 0: reflector from column 0, segment sums of y_0 = A22 v_0
-    double2 t;
-    double beta;
-    {
-        const int L = n - 1;
-        for (int k = threadIdx.x; k < L; k += blockDim.x) v[k] = __ldcg(A + 1 + k);
-        __syncthreads();
-        make_reflector(v, L, red, t, beta);
-        if (blockIdx.x == 0) {
-            for (int k = threadIdx.x; k < L; k += blockDim.x) V[1 + k] = v[k];
-            if (threadIdx.x == 0) {
-                tau[0] = t;
-                e[0] = beta;
-                d[0] = __ldcg(A).x;
-            }
-        }
-        const int nseg = (L + SEG - 1) / SEG;
-        for (int u = gwarp; u < L * nseg; u += nwarps) {
-            const int k = u / nseg, sg = u - k * nseg;
-            const double2* col = A + 1 + (long)(1 + k) * n;
-            const int c0 = sg * SEG + lane;
-            double2 a[PER];
+    if (in_smem)
+        for (int s = 0; s < nown; ++s)
+            for (int r = tid; r < n; r += HT) cols[s * cstr + r] = A[(long)(bid + s * nb) * n + r];
+    // x: the column to eliminate (rows > i), as registers; v, w of this step, vp, of the last
+    double2 v[PER], w[PER], x[PER];
 #pragma unroll
-            for (int q = 0; q < PER; ++q) {
-                const int cc = c0 + 32 * q;
-                a[q] = cc < L ? __ldcg(col + cc) : make_double2(0.0, 0.0);
-            }
-            double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-            for (int q = 0; q < PER; ++q) {
-                const int cc = c0 + 32 * q;
-                if (cc < L) acc = cadd(acc, cmulc(a[q], v[cc]));
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-            }
-            if (lane == 0) Yp[(long)sg * n + k] = acc;
-        }
-        if (!grid_barrier(bar, nb, err)) return;
+    for (int q = 0; q < PER; ++q) {
+        const int r = tid + q * HT;
+        x[q] = r < n ? __ldcg(A + r) : make_double2(0.0, 0.0);
+        v[q] = w[q] = make_double2(0.0, 0.0);
     }
-    for (int i = 0; i < n - 1; ++i) {
-        const int L = n - i - 1;  // A22 of step i: rows/columns i + 1 .. n - 1
-        const int nseg = (L + SEG - 1) / SEG;
-        // w_i from the segment sums of y_i
-        double sp = 0;
-        for (int k = threadIdx.x; k < L; k += blockDim.x) {
-            double2 y = __ldcg(Yp + k);
-            for (int sg = 1; sg < nseg; ++sg) y = cadd(y, __ldcg(Yp + (long)sg * n + k));
-            w[k] = y;
-            sp += v[k].x * y.x + v[k].y * y.y;
+    if (bid == 0 && tid == 0) d[0] = x[0].x;
+    for (int i = 0;; ++i) {
+        // reflector v_i from x (rows i + 1 ..); every thread derives the scalars itself
+        double ss = 0;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int r = tid + q * HT;
+            if (r == i + 1) head[0] = x[q];
+            if ((r | 31) < i + 2 || (r & ~31) >= n) continue;  // warp-uniform
+            if (r >= i + 2 && r < n) ss = fma(x[q].x, x[q].x, fma(x[q].y, x[q].y, ss));
         }
-        const double sv = block_sum(sp, red);
-        const double h = 0.5 * (t.x * t.x + t.y * t.y) * sv;
-        for (int k = threadIdx.x; k < L; k += blockDim.x) w[k] = csub(cmul(t, w[k]), cscale(v[k], h));
-        __syncthreads();
-        const double2 v0c = zconj(v[0]), w0c = zconj(w[0]);
-        if (L == 1) {  // last step: the remaining 1 x 1 block
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                const double2 a = __ldcg(A + (n - 1) + (long)(n - 1) * n);
-                d[n - 1] = csub(a, cadd(cmul(v[0], w0c), cmul(w[0], v0c))).x;
+        const double xn2 = ht_sum<HT>(ss, red[0]);
+        const double2 al = head[0];
+        double2 t = make_double2(0.0, 0.0), sc = t;
+        double beta = al.x;
+        if (!(xn2 == 0.0 && al.y == 0.0)) {  // else nothing to eliminate: H = I
+            const double s2 = fma(al.x, al.x, fma(al.y, al.y, xn2));
+            double ib, id, dx;
+            if (s2 > 0x1p-900 && s2 < 0x1p+900) {
+                const double rs = newton_rsqrt(s2);
+                ib = -copysign(rs, al.x);
+                beta = s2 * ib;  // -sign(Re alpha) sqrt(s2)
+                dx = al.x - beta;
+                id = newton_rcp(fma(dx, dx, al.y * al.y));
+            } else {
+                beta = -copysign(sqrt(s2), al.x);
+                ib = 1.0 / beta;
+                dx = al.x - beta;
+                id = 1.0 / fma(dx, dx, al.y * al.y);
             }
-            break;
+            t = make_double2(-dx * ib, -al.y * ib);
+            sc = make_double2(dx * id, -al.y * id);  // 1 / (alpha - beta)
         }
-        // updated column i + 1 (rows i + 1 .. n - 1) and the reflector v_{i+1}
-        const double2* colx = A + (i + 1) + (long)(i + 1) * n;
-        for (int k = threadIdx.x; k < L; k += blockDim.x)
-            vn[k] = csub(__ldcg(colx + k), cadd(cmul(v[k], w0c), cmul(w[k], v0c)));
-        __syncthreads();
-        const double dnext = vn[0].x;
-        const int L1 = L - 1;  // A22 of step i + 1
-        double2 tn;
-        double bn;
-        make_reflector(vn + 1, L1, red, tn, bn);
-        if (blockIdx.x == 0) {
-            for (int k = threadIdx.x; k < L1; k += blockDim.x) V[(i + 2 + k) + (long)(i + 1) * n] = vn[1 + k];
-            if (threadIdx.x == 0) {
-                tau[i + 1] = tn;
-                e[i + 1] = bn;
-                d[i + 1] = dnext;
+        // v_i into x; the registers v keep v_{i-1} for the update below
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int r = tid + q * HT;
+            if (r == i + 1) {
+                x[q] = make_double2(1.0, 0.0);
+            } else if (r > i + 1 && r < n) {
+                x[q] = make_double2(fma(x[q].x, sc.x, -x[q].y * sc.y), fma(x[q].x, sc.y, x[q].y * sc.x));
+            } else {
+                x[q] = make_double2(0.0, 0.0);
             }
+            if (bid == 0 && r > i && r < n) V[r + (long)i * n] = x[q];
         }
-        // fused units: update A22_{i+1} = rows/columns i + 2 .. n - 1 by step i's rank-2
-        // term, then the segment sums of y_{i+1} = A22_{i+1} v_{i+1}
-        const int nseg1 = (L1 + SEG - 1) / SEG;
-        const double2* vv = vn + 1;
-        for (int u = gwarp; u < L1 * nseg1; u += nwarps) {
-            const int cidx = u / nseg1, sg = u - cidx * nseg1;
-            double2* col = A + (i + 2) + (long)(i + 2 + cidx) * n;
-            const double2 vc = zconj(v[1 + cidx]), wc = zconj(w[1 + cidx]);
-            const int r0 = sg * SEG + lane;
-            double2 a[PER];
+        if (bid == 0 && tid == 0) {
+            tau[i] = t;
+            e[i] = beta;
+        }
+        // own columns j > i: the rank-2 term of step i - 1, then y_i[j] = <column j, v_i>
+        const int s0 = (i + 1 - bid + nb - 1) / nb;  // first owned column beyond i
+        auto column = [&](int s) {
+            const int j = bid + s * nb;
+            double2* col = cols + s * cstr;
+            double2 vj = make_double2(0.0, 0.0), wj = vj, acc = vj;
+            if (i > 0) vj = sv[j], wj = sw[j];
 #pragma unroll
             for (int q = 0; q < PER; ++q) {
-                const int r = r0 + 32 * q;
-                if (r < L1) a[q] = __ldcg(col + r);
-            }
-            double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-            for (int q = 0; q < PER; ++q) {
-                const int r = r0 + 32 * q;
-                if (r < L1) {
-                    const double2 nv = csub(a[q], cadd(cmul(v[1 + r], wc), cmul(w[1 + r], vc)));
-                    col[r] = nv;
-                    acc = cadd(acc, cmulc(nv, vv[r]));
+                const int r = tid + q * HT;
+                if ((r | 31) <= i || (r & ~31) >= n) continue;  // warp-uniform
+                if (r > i && r < n) {
+                    double2 a = col[r];
+                    if (i > 0) {  // a -= v conj(wj) + w conj(vj)
+                        a.x = fma(-v[q].x, wj.x, fma(-v[q].y, wj.y, fma(-w[q].x, vj.x, fma(-w[q].y, vj.y, a.x))));
+                        a.y = fma(v[q].x, wj.y, fma(-v[q].y, wj.x, fma(w[q].x, vj.y, fma(-w[q].y, vj.x, a.y))));
+                        col[r] = a;
+                    }
+                    if (j == i + 1) {
+                        publish(&C[(long)i * n + r].x, a.x);
+                        publish(&C[(long)i * n + r].y, a.y);
+                    }
+                    acc.x = fma(a.x, x[q].x, fma(a.y, x[q].y, acc.x));
+                    acc.y = fma(a.x, x[q].y, fma(-a.y, x[q].x, acc.y));
                 }
             }
-            for (int o = 16; o > 0; o >>= 1) {
-                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-            }
-            if (lane == 0) Yp[(long)sg * n + cidx] = acc;
+            return acc;
+        };
+        // warp sums of two columns at a time: lanes below 16 take the first, the others the
+        // second, then every eight lanes the real or the imaginary parts
+        for (int s = s0; s < nown; s += 2) {
+            const double2 a0 = column(s);
+            const double2 a1 = s + 1 < nown ? column(s + 1) : make_double2(0.0, 0.0);
+            const bool up = lane & 16;
+            const double kx = up ? a1.x : a0.x, ky = up ? a1.y : a0.y;
+            const double sx = up ? a0.x : a1.x, sy = up ? a0.y : a1.y;
+            const double px = kx + __shfl_xor_sync(0xffffffffu, sx, 16);
+            const double py = ky + __shfl_xor_sync(0xffffffffu, sy, 16);
+            const bool im = lane & 8;
+            double p = (im ? py : px) + __shfl_xor_sync(0xffffffffu, im ? px : py, 8);
+            for (int o = 4; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+            const int sc_ = s + (lane >> 4);
+            if ((lane & 7) == 0 && sc_ < nown)
+                reinterpret_cast<double*>(part + sc_ * (HT / 32) + wp)[(lane >> 3) & 1] = p;
         }
-        // the next step works with v_{i+1}
         __syncthreads();
-        for (int k = threadIdx.x; k < L1; k += blockDim.x) v[k] = vv[k];
-        t = tn;
-        if (!grid_barrier(bar, nb, err)) return;
+        for (int q = tid; q < 2 * (nown - s0); q += HT) {
+            const int s = s0 + (q >> 1), c = q & 1;
+            const double* ps = reinterpret_cast<const double*>(part + s * (HT / 32)) + c;
+            publish(reinterpret_cast<double*>(Y + (long)i * n + bid + s * nb) + c,
+                    HT == 128 ? (ps[0] + ps[2]) + (ps[4] + ps[6])
+                              : ((ps[0] + ps[2]) + (ps[4] + ps[6])) + ((ps[8] + ps[10]) + (ps[12] + ps[14])));
+        }
+        // everybody's y_i and column i + 1
+        double2 y[PER], c[PER];
+        {
+            long long it = 0;
+            bool more = true;
+            while (more) {
+                more = false;
+#pragma unroll
+                for (int q = 0; q < PER; ++q) {
+                    const int r = tid + q * HT;
+                    if (r > i && r < n) {
+                        y[q] = peek(Y + (long)i * n + r);
+                        c[q] = peek(C + (long)i * n + r);
+                    } else {
+                        y[q] = c[q] = make_double2(0.0, 0.0);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < PER; ++q) more = more || is_empty(y[q]) || is_empty(c[q]);
+                if (more && (++it > BAR_LIMIT || ((it & 1023) == 0 && *(volatile int*)err))) {
+                    atomicExch(err, 1);
+                    gave_up = 1;
+                    break;
+                }
+            }
+        }
+        double sp = 0;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int r = tid + q * HT;
+            if ((r | 31) <= i || (r & ~31) >= n) continue;
+            if (r == i + 1) head[1] = y[q];
+            sp = fma(x[q].x, y[q].x, fma(x[q].y, y[q].y, sp));
+        }
+        const double h = 0.5 * fma(t.x, t.x, t.y * t.y) * ht_sum<HT>(sp, red[1]);
+        if (gave_up) return;  // block-uniform: set before the barrier in ht_sum
+        const double2 y0 = head[1];
+        const double2 w0 = make_double2(fma(t.x, y0.x, fma(-t.y, y0.y, -h)), fma(t.x, y0.y, t.y * y0.x));
+        // v <- v_i, w <- w_i = t y - h v, x <- column i + 1 minus its rank-2 term (v[0] = 1)
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int r = tid + q * HT;
+            if ((r | 31) <= i || (r & ~31) >= n) continue;
+            v[q] = x[q];
+            w[q] = make_double2(fma(t.x, y[q].x, fma(-t.y, y[q].y, -h * v[q].x)),
+                                fma(t.x, y[q].y, fma(t.y, y[q].x, -h * v[q].y)));
+            x[q].x = c[q].x - fma(v[q].x, w0.x, fma(v[q].y, w0.y, w[q].x));
+            x[q].y = c[q].y - fma(v[q].y, w0.x, fma(-v[q].x, w0.y, w[q].y));
+            if (r > i && r < n) {
+                sv[r] = v[q];
+                sw[r] = w[q];
+                if (r == i + 1 && bid == 0) d[i + 1] = x[q].x;
+            }
+        }
+        if (i == n - 2) return;
+        // sv, sw are read after the barrier in the next ht_sum
     }
 }
 
@@ -441,41 +520,50 @@ hetrd_kernel(int n, double2* A, double2* V, double2* tau, double* d, double* e, 
 // principal minors p_j = (d_j - x) p_{j-1} - e_{j-1}^2 p_{j-2} (p_{-1} = 1),
 // carried with exact power-of-two rescaling (no division); a zero minor counts
 // as a change of sign, the role of LAPACK's pivmin in the ratio form.
+// FP64 instructions are what a step costs (three here), so signs, zero tests and the range
+// checks (every fourth step: a step changes the magnitude by far less than 2^100 up, and a
+// minor that falls out of range at the bottom has lost its weight) are taken on the high words.
 __device__ __forceinline__ int sturm_count(const double* d, const double* e2, int n, double x, double) {
     const double big = 0x1p+500, small = 0x1p-500;
     double pm = 1.0, p = d[0] - x;
     int cnt = !(p > 0.0);
     if (p == 0.0) p = -small;
+#pragma unroll 4
     for (int j = 1; j < n; ++j) {
-        double q = (d[j] - x) * p - e2[j - 1] * pm;
-        if (q == 0.0) q = p > 0.0 ? -small : small;
-        cnt += (q > 0.0) != (p > 0.0);
+        double q = fma(d[j] - x, p, -(e2[j - 1] * pm));
+        const int hp = __double2hiint(p), hq = __double2hiint(q);
+        if ((((unsigned)hq << 1) | (unsigned)__double2loint(q)) == 0) {
+            q = hp >= 0 ? -small : small;
+            cnt += 1;
+        } else {
+            cnt += (unsigned)(hq ^ hp) >> 31;
+        }
         pm = p;
         p = q;
-        const double ap = fabs(p);
-        if (ap > big) {
-            p *= small;
-            pm *= small;
-        } else if (ap < small && fabs(pm) < small) {
-            p *= big;
-            pm *= big;
+        if ((j & 3) == 3) {
+            const int ep = (__double2hiint(p) >> 20) & 0x7ff, em = (__double2hiint(pm) >> 20) & 0x7ff;
+            if (ep > 1023 + 400) {
+                p *= small;
+                pm *= small;
+            } else if (max(ep, em) < 1023 - 400) {
+                p *= big;
+                pm *= big;
+            }
         }
     }
     return cnt;
 }
 
-// e2 = e^2 and the Gershgorin interval, pivmin (one block)
-__global__ void tri_prep_kernel(const double* d, const double* e, double* e2, int n, double* info3) {
+// T scaled by a power of two to a norm of about one (ds, e2 = scaled e squared) for the counts,
+// its Gershgorin interval and pivmin; info3[3]: the norm of T, [4]: the factor back (one block)
+__global__ void tri_prep_kernel(const double* d, const double* e, double* ds, double* e2, int n, double* info3) {
     __shared__ double lo_s[256], hi_s[256], em_s[256];
     double lo = 1e300, hi = -1e300, em = 0;
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         const double a = j > 0 ? fabs(e[j - 1]) : 0.0, b = j < n - 1 ? fabs(e[j]) : 0.0;
         lo = fmin(lo, d[j] - a - b);
         hi = fmax(hi, d[j] + a + b);
-        if (j < n - 1) {
-            e2[j] = e[j] * e[j];
-            em = fmax(em, e2[j]);
-        }
+        if (j < n - 1) em = fmax(em, fabs(e[j]));
     }
     lo_s[threadIdx.x] = lo;
     hi_s[threadIdx.x] = hi;
@@ -489,13 +577,22 @@ __global__ void tri_prep_kernel(const double* d, const double* e, double* e2, in
         }
         __syncthreads();
     }
+    const double tnorm = fmax(fabs(lo_s[0]), fabs(hi_s[0]));
+    int ex = 0;
+    if (tnorm > 0 && isfinite(tnorm)) frexp(tnorm, &ex);
+    ex = min(max(ex, -1000), 1000);
+    const double sc = ldexp(1.0, -ex);
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        ds[j] = d[j] * sc;
+        if (j < n - 1) e2[j] = (e[j] * sc) * (e[j] * sc);
+    }
     if (threadIdx.x == 0) {
-        const double tnorm = fmax(fabs(lo_s[0]), fabs(hi_s[0]));
-        const double pad = 2.0 * DBL_EPSILON * tnorm + 1e-300;
-        info3[0] = lo_s[0] - pad;
-        info3[1] = hi_s[0] + pad;
-        info3[2] = fmax(1e-300, DBL_MIN * fmax(1.0, em_s[0]));  // pivmin
+        const double pad = 2.0 * DBL_EPSILON * (tnorm * sc) + 1e-300;
+        info3[0] = lo_s[0] * sc - pad;
+        info3[1] = hi_s[0] * sc + pad;
+        info3[2] = fmax(1e-300, DBL_MIN * fmax(1.0, (em_s[0] * sc) * (em_s[0] * sc)));  // pivmin
         info3[3] = tnorm;
+        info3[4] = ldexp(1.0, ex);
     }
 }
 
@@ -520,7 +617,7 @@ __global__ void tri_bisect_kernel(const double* d, const double* e2, int n, int 
         a = na_;
         b = f < 31 ? nb_ : b;
     }
-    if (lane == 0) w[k] = 0.5 * (a + b);
+    if (lane == 0) w[k] = 0.5 * (a + b) * info3[4];
 }
 
 // ------------------------------------------------------------------ tridiagonal eigenvectors
@@ -534,9 +631,10 @@ __global__ void tri_bisect_kernel(const double* d, const double* e2, int n, int 
 // a cluster.  Lane 0 runs the elimination and the substitutions (sequential in
 // the position) on shared-memory copies of T, of the factors and of the
 // vector; all lanes run the Gram-Schmidt steps and the norms.  z: [n][m] real
-// (position-major).  Dynamic shared memory: 8 n doubles.
+// (position-major) and, complex, in Z.  Dynamic shared memory: 8 n doubles.
 __global__ void __launch_bounds__(32) tri_invit_kernel(const double* d, const double* e, int n, int m,
-                                                       const double* w, const double* info3, double* z) {
+                                                       const double* w, const double* info3, double* z,
+                                                       double2* Z, int ldz) {
     extern __shared__ __align__(16) double tsm[];
     double* dd = tsm;          // diagonal of T
     double* ee = dd + n;       // off-diagonal of T (ee[n - 1] = 0)
@@ -587,16 +685,20 @@ __global__ void __launch_bounds__(32) tri_invit_kernel(const double* d, const do
                 }
             }
             ri[n - 1] = p0 == 0.0 ? sep : p0;
-            for (int i = 0; i < n - 1; ++i) {
-                const double u = ri[i];
-                if (fabs(u) < sep) ri[i] = u < 0 ? -sep : sep;
-            }
             // start vector: a fixed pseudo-random sequence per index
             unsigned int st = 2654435761u * (unsigned int)(k + 1) + 12345u;
             for (int i = 0; i < n; ++i) {
                 st = st * 1664525u + 1013904223u;
                 zv[i] = 0.5 + (double)(st >> 8) * (1.0 / 16777216.0);
             }
+        }
+        __syncwarp();
+        // small pivots raised to eps ||T||, then their reciprocals (a division per position and
+        // sweep on lane 0 alone would be the longest chain of the iteration)
+        for (int i = lane; i < n; i += 32) {
+            double u = ri[i];
+            if (fabs(u) < sep) u = u < 0 ? -sep : sep;
+            ri[i] = 1.0 / u;
         }
         __syncwarp();
         for (int it = 0; it < 4; ++it) {
@@ -615,10 +717,10 @@ __global__ void __launch_bounds__(32) tri_invit_kernel(const double* d, const do
                 }
                 zv[n - 1] = xi;
                 // back substitution with the three diagonals of U
-                double x2 = 0.0, x1 = zv[n - 1] / ri[n - 1];
+                double x2 = 0.0, x1 = zv[n - 1] * ri[n - 1];
                 zv[n - 1] = x1;
                 for (int i = n - 2; i >= 0; --i) {
-                    const double x0 = (zv[i] - u1[i] * x1 - u2[i] * x2) / ri[i];
+                    const double x0 = fma(-u1[i], x1, fma(-u2[i], x2, zv[i])) * ri[i];
                     zv[i] = x0;
                     x2 = x1;
                     x1 = x0;
@@ -640,69 +742,51 @@ __global__ void __launch_bounds__(32) tri_invit_kernel(const double* d, const do
             for (int i = lane; i < n; i += 32) zv[i] *= inv;
             __syncwarp();
         }
-        for (int i = lane; i < n; i += 32) ZV(k, i) = zv[i];
+        for (int i = lane; i < n; i += 32) {
+            ZV(k, i) = zv[i];
+            Z[i + (long)k * ldz] = make_double2(zv[i], 0.0);
+        }
         __syncwarp();
     }
 #undef ZV
 }
 
 // ------------------------------------------------------------------ back-transformation
-// Z = Q z with Q = H_0 ... H_{n-2}, applied in blocks of NBLK reflectors from
-// the last block to the first: Q_b = H_j0 ... H_j1-1 = I - V_b T_b V_b^H
-// (compact WY form; T_b upper triangular, T_jj = tau_j,
-// T[0:j, j] = -tau_j T[0:j, 0:j] (V_b^H v_j)[0:j]), Z <- Z - V_b (T_b (V_b^H Z)).
+// Z = Q z with Q = H_0 ... H_{n-2}, applied in blocks of IB reflectors from the last block
+// to the first: Q_b = H_j0 ... H_j1-1 = I - V_b T_b V_b^H (compact WY form, T_b upper
+// triangular), Z <- Z - V_b (T_b (V_b^H Z)).  T_b^-1 = strictly upper part of V_b^H V_b plus
+// diag(1 / tau) (Joffrain, Low, Quintana-Orti, van de Geijn and Van Zee, 2006), so T_b^H is
+// the inverse of a lower triangular matrix and comes from the kernel of the triangular
+// solves.  A reflector with tau = 0 (H = I) gets a zero column and the diagonal entry 1.
+// (Blocks of 32 with a column recurrence for T, and V_b^H V_b from warp-wide dot products on
+// the FP64 units, took 9.2 ms at n = 816, m = 272.)
 
-// z (position-major [n][m], real) -> Z (column-major, complex)
-__global__ void tri_z_to_Z_kernel(int n, int m, const double* z, double2* Z, int ldz) {
-    long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (t >= (long)n * m) return;
-    const int i = (int)(t % n), j = (int)(t / n);
-    Z[i + (long)j * ldz] = make_double2(z[(long)i * m + j], 0.0);
+// V[:, j] <- 0 where tau_j = 0
+__global__ void wy_zero_kernel(int n, double2* V, const double2* tau) {
+    const int j = blockIdx.x;
+    if (tau[j].x != 0.0 || tau[j].y != 0.0) return;
+    for (int r = threadIdx.x; r < n; r += blockDim.x) V[r + (long)j * n] = make_double2(0.0, 0.0);
 }
-
-// T_b of every block of reflectors at once: block b (reflectors j0 = b NBLK ..)
-// forms G = V_b^H V_b (rows j0 + 1 .. n - 1) and then T_b column by column;
-// T_b goes to T + b NBLK NBLK (ld NBLK).
-__global__ void __launch_bounds__(256) wy_t_kernel(int n, const double2* V, const double2* tau, double2* T) {
-    __shared__ double2 Ts[NBLK][NBLK + 1];
-    __shared__ double2 Gs[NBLK][NBLK + 1];
-    __shared__ double2 ts[NBLK];
-    const int j0 = blockIdx.x * NBLK, nbk = min(NBLK, n - 1 - j0), r0 = j0 + 1;
-    const double2* Vb = V + (long)j0 * n;
-    // G[p][q] = sum_rows conj(V[row][j0 + p]) V[row][j0 + q]: a warp per (p, q) entry
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    for (int e = wp; e < nbk * nbk; e += 8) {
-        const int p = e % nbk, q = e / nbk;
-        double2 acc = make_double2(0.0, 0.0);
-        for (int row = r0 + lane; row < n; row += 32)
-            acc = cadd(acc, cmulc(Vb[row + (long)p * n], Vb[row + (long)q * n]));
-        for (int o = 16; o > 0; o >>= 1) {
-            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-        }
-        if (lane == 0) Gs[p][q] = acc;
-    }
-    if (threadIdx.x < nbk) ts[threadIdx.x] = tau[j0 + threadIdx.x];
-    __syncthreads();
-    T += (size_t)blockIdx.x * NBLK * NBLK;
-    const int r = threadIdx.x;
-    for (int j = 0; j < nbk; ++j) {
-        // column j: T[r][j] = -tau_j sum_{q<j} T[r][q] G[q][j] for r < j; T[j][j] = tau_j
-        double2 v = make_double2(0.0, 0.0);
-        if (r < j) {
-            for (int q = r; q < j; ++q) v = cadd(v, cmul(Ts[r][q], Gs[q][j]));
-            v = cmul(make_double2(-ts[j].x, -ts[j].y), v);
-        } else if (r == j) {
-            v = ts[j];
-        }
-        __syncthreads();
-        if (r < nbk) Ts[r][j] = v;
-        __syncthreads();
-    }
-    for (int j = 0; j < nbk; ++j)
-        if (r < nbk) T[r + (long)j * nbk] = r <= j ? Ts[r][j] : make_double2(0.0, 0.0);
+// M (lower, ld IB): strictly lower part of G = V_b^H V_b (which is the conjugate transpose of
+// its strictly upper part), diagonal 1 / conj(tau) scaled to 1: row r of M times conj(tau_r)
+// keeps tri_inv_kernel's real unit diagonal; the inverse's columns are scaled back in wy_scale
+__global__ void wy_m_kernel(int nbk, double2* G, const double2* tau) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nbk * nbk) return;
+    const int r = t % nbk, c = t / nbk;
+    double2 tr = zconj(tau[r]);
+    if (tr.x == 0.0 && tr.y == 0.0) tr = make_double2(1.0, 0.0);
+    double2* g = G + r + (long)c * IB;
+    *g = r > c ? cmul(tr, *g) : make_double2(r == c ? 1.0 : 0.0, 0.0);
 }
-
+// rows of X (b x m): X[r] *= tau_r (1 where tau = 0)
+__global__ void wy_scale_kernel(int b, int m, double2* X, const double2* tau) {
+    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (t >= (long)b * m) return;
+    const double2 tr = tau[t % b];
+    if (tr.x == 0.0 && tr.y == 0.0) return;
+    X[t] = cmul(X[t], tr);
+}
 
 inline int cdiv(long a, long b) { return (int)((a + b - 1) / b); }
 
@@ -778,51 +862,83 @@ void dense_gemm(fs_ctx* c, int opA, int opB, int M, int N, int K, double alpha, 
     dense_gemm_mat(c, M, N, K, alpha, op_a(opA, A, lda), op_b(opB, B, ldb), beta, OzDst{C, 1, ldc}, 0, 0);
 }
 
-// Cholesky of the lower triangle of A (n x n, ld lda); squared pivots to piv
-// (device, may be null).  Returns the LAPACK info (0, or the first failing
-// column + 1).  Synchronises the context's stream.
-int dense_potrf(fs_ctx* c, int n, double2* A, int lda, double* piv) {
+// Cholesky of the lower triangle of A (n x n, ld lda); squared pivots to piv (device, may be
+// null); info (device int, zeroed here): 0, or the first failing column + 1 as LAPACK's.
+// Blocks of 32 within panels of PB columns; what a panel leaves to the columns beyond it is
+// one product of PB k (on the tensor cores from 6e7 flops on).
+static void potrf_async(fs_ctx* c, int n, double2* A, int lda, double* piv, int* info) {
     ProfScope ps(c, KS_SUB_POTRF, 0.0, 8.0 * n * (double)n * n / 3.0);
-    DenseWork& D = c->dense;
-    D.info.ensure(sizeof(int));
-    int* info = D.info.as<int>();
+    constexpr int PB = 128;
     FS_CUDA(cudaMemsetAsync(info, 0, sizeof(int), c->stream));
-    for (int j0 = 0; j0 < n; j0 += NBLK) {
-        const int b = std::min(NBLK, n - j0);
-        potrf_diag_kernel<<<1, NBLK * NBLK, 0, c->stream>>>(A, lda, j0, b, piv, info);
-        const int rest = n - j0 - b;
-        if (rest > 0) {
-            potrf_panel_kernel<<<cdiv((long)rest * 32, 256), 256, 0, c->stream>>>(A, lda, n, j0, b);
-            // trailing update of the lower triangle (the upper one is never read)
+    for (int p0 = 0; p0 < n; p0 += PB) {
+        const int pe = std::min(n, p0 + PB);
+        for (int j0 = p0; j0 < pe; j0 += NBLK) {
+            const int b = std::min(NBLK, pe - j0);
+            potrf_diag_kernel<<<1, NBLK * NBLK, 0, c->stream>>>(A, lda, j0, b, piv, info);
+            const int rest = n - j0 - b;
+            if (rest <= 0) continue;
+            potrf_panel_kernel<<<cdiv((long)rest * 32, 128), 128, 0, c->stream>>>(A, lda, n, j0, b);
+            // the panel's own remaining columns (lower triangle; the upper one is never read)
+            const int own = pe - j0 - b;
             const double2* pan = A + j0 + b + (long)j0 * lda;
-            dense_gemm_mat(c, rest, rest, b, -1.0, op_a(0, pan, lda), op_b(1, pan, lda), 1.0,
-                           OzDst{A + j0 + b + (long)(j0 + b) * lda, 1, lda}, 0, 1);
+            if (own > 0)
+                dense_gemm_mat(c, rest, own, b, -1.0, op_a(0, pan, lda), op_b(1, pan, lda), 1.0,
+                               OzDst{A + j0 + b + (long)(j0 + b) * lda, 1, lda}, 0, 1);
+        }
+        const int rest = n - pe;
+        if (rest > 0) {
+            const double2* pan = A + pe + (long)p0 * lda;
+            const bool big = oz_worth(rest, rest, pe - p0);
+            dense_gemm_mat(c, rest, rest, pe - p0, -1.0, op_a(0, pan, lda), op_b(1, pan, lda), 1.0,
+                           OzDst{A + pe + (long)pe * lda, 1, lda}, 0, big ? 0 : 1);
         }
     }
     FS_CUDA(cudaGetLastError());
+}
+
+// The same; returns the info.  Synchronises the context's stream.
+int dense_potrf(fs_ctx* c, int n, double2* A, int lda, double* piv) {
+    DenseWork& D = c->dense;
+    D.info.ensure(2 * sizeof(int));
+    potrf_async(c, n, A, lda, piv, D.info.as<int>());
     int h = 0;
-    FS_CUDA(cudaMemcpyAsync(&h, info, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    FS_CUDA(cudaMemcpyAsync(&h, D.info.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     FS_CUDA(cudaStreamSynchronize(c->stream));
     return h;
 }
 
-// B <- L^-1 B (conj = 0) or L^-H B (conj = 1); L lower n x n (ld lda), B n x ncols (ld ldb)
-void dense_trsm(fs_ctx* c, int conj, int n, int ncols, const double2* L, int lda, double2* B, int ldb) {
+// Inverses of the diagonal blocks of L (lower n x n) for the following dense_trsm calls with the same L
+static void tri_inverses(fs_ctx* c, int n, const double2* L, int lda) {
+    DenseWork& D = c->dense;
+    D.linv.ensure((size_t)cdiv(n, IB) * IB * IB * sizeof(double2));
+    tri_inv_kernel<<<cdiv((long)cdiv(n, IB) * IB, 4), 128, 0, c->stream>>>(L, lda, n, D.linv.as<double2>());
+    FS_CUDA(cudaGetLastError());
+}
+
+// B <- L^-1 B (conj = 0) or L^-H B (conj = 1); L lower n x n (ld lda), B n x ncols (ld ldb).
+// Blocks of IB rows: x_b = inv(L_bb) b_b, then the rest of B minus its product with x_b.
+// fresh = false: the inverses of the last call's L are the ones of this L.
+void dense_trsm(fs_ctx* c, int conj, int n, int ncols, const double2* L, int lda, double2* B, int ldb, bool fresh) {
     if (n <= 0 || ncols <= 0) return;
     ProfScope ps(c, KS_SUB_TRSM, 0.0, 4.0 * n * (double)n * ncols);
-    const int nblk = cdiv(n, NBLK);
+    if (fresh) tri_inverses(c, n, L, lda);
+    DenseWork& D = c->dense;
+    D.xb.ensure((size_t)IB * ncols * sizeof(double2));
+    double2* X = D.xb.as<double2>();
+    const int nblk = cdiv(n, IB);
     for (int q = 0; q < nblk; ++q) {
         const int bi = conj ? nblk - 1 - q : q;
-        const int j0 = bi * NBLK, b = std::min(NBLK, n - j0);
-        trsm_diag_kernel<<<cdiv((long)ncols * 32, 256), 256, 0, c->stream>>>(L, lda, j0, b, B, ldb, ncols, conj);
+        const int j0 = bi * IB, b = std::min(IB, n - j0);
+        dense_gemm(c, conj ? 1 : 0, 0, b, ncols, b, 1.0, D.linv.as<double2>() + (size_t)bi * IB * IB, IB, B + j0, ldb,
+                   0.0, X, b);
+        FS_CUDA(cudaMemcpy2DAsync(B + j0, ldb * sizeof(double2), X, b * sizeof(double2), b * sizeof(double2), ncols,
+                                  cudaMemcpyDeviceToDevice, c->stream));
         if (!conj) {
             const int rest = n - j0 - b;
-            if (rest > 0)
-                dense_gemm(c, 0, 0, rest, ncols, b, -1.0, L + j0 + b + (long)j0 * lda, lda, B + j0, ldb, 1.0,
-                           B + j0 + b, ldb);
-        } else if (j0 > 0) {
+            dense_gemm(c, 0, 0, rest, ncols, b, -1.0, L + j0 + b + (long)j0 * lda, lda, X, b, 1.0, B + j0 + b, ldb);
+        } else {
             // B[0:j0] -= (L[j0:j0+b, 0:j0])^H X_b
-            dense_gemm(c, 1, 0, j0, ncols, b, -1.0, L + j0, lda, B + j0, ldb, 1.0, B, ldb);
+            dense_gemm(c, 1, 0, j0, ncols, b, -1.0, L + j0, lda, X, b, 1.0, B, ldb);
         }
     }
     FS_CUDA(cudaGetLastError());
@@ -844,29 +960,40 @@ void dense_heev(fs_ctx* c, int n, double2* A, int m, double* w, double2* Z, int 
     D.d.ensure((size_t)n * sizeof(double));
     D.e.ensure((size_t)n * sizeof(double));
     D.e2.ensure((size_t)n * sizeof(double));
-    D.Y.ensure((size_t)((n + SEG - 1) / SEG) * n * sizeof(double2));
+    D.Y.ensure((size_t)2 * n * n * sizeof(double2));  // a row of y and a row of columns per step
     D.z.ensure((size_t)n * m * sizeof(double));
-    D.info3.ensure(4 * sizeof(double));
-    D.bar.ensure(2 * sizeof(unsigned int));
+    D.info3.ensure(5 * sizeof(double));
+    D.ds.ensure((size_t)n * sizeof(double));
     int dev = 0, nsm = 0;
     FS_CUDA(cudaGetDevice(&dev));
     FS_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const size_t smem = (size_t)3 * n * sizeof(double2);
+    // four warps up to n = 1024 (8 rows a thread), eight beyond
+    const int ht = n <= 1024 ? 128 : 256;
+    const void* hk = n <= 128    ? (const void*)hetrd_kernel<128, 1>
+                     : n <= 256  ? (const void*)hetrd_kernel<128, 2>
+                     : n <= 512  ? (const void*)hetrd_kernel<128, 4>
+                     : n <= 1024 ? (const void*)hetrd_kernel<128, 8>
+                                 : (const void*)hetrd_kernel<256, 8>;
     if (!D.attr_set) {
-        FS_CUDA(cudaFuncSetAttribute((const void*)hetrd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     3 * FS_DENSE_MAX_N * (int)sizeof(double2)));
+        for (const void* k : {(const void*)hetrd_kernel<128, 1>, (const void*)hetrd_kernel<128, 2>,
+                              (const void*)hetrd_kernel<128, 4>, (const void*)hetrd_kernel<128, 8>,
+                              (const void*)hetrd_kernel<256, 8>})
+            FS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, HETRD_SMEM));
         FS_CUDA(cudaFuncSetAttribute((const void*)tri_invit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      8 * FS_DENSE_MAX_N * (int)sizeof(double)));
         D.attr_set = true;
     }
-    int per_sm = 0;
-    FS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hetrd_kernel, 256, smem));
-    // enough warps for the (column, segment) units, at most one block per SM
-    const int nblocks = std::max(1, std::min({nsm, nsm * std::max(per_sm, 1), (n + 3) / 4}));
+    // a block per column, at most one per SM; the columns in shared memory when they fit
+    // (n <= 1216 on 152 SMs)
+    const int nblocks = std::max(1, std::min(nsm, n - 1));
+    const size_t vecs = (size_t)2 * n * sizeof(double2) + (size_t)cdiv(n, nblocks) * (ht / 32) * sizeof(double2);
+    const size_t own = (size_t)cdiv(n, nblocks) * n * sizeof(double2);
+    int in_smem = vecs + own <= (size_t)HETRD_SMEM;
+    const size_t smem = vecs + (in_smem ? own : 0);
     {
     ProfScope ps_h(c, KS_SUB_HETRD, 0.0, 16.0 * n * (double)n * n / 3.0);
     hermitize_kernel<<<cdiv((long)n * n, 256), 256, 0, c->stream>>>(A, n);
-    FS_CUDA(cudaMemsetAsync(D.bar.p, 0, 2 * sizeof(unsigned int), c->stream));
+    FS_CUDA(cudaMemsetAsync(D.Y.p, 0xff, (size_t)2 * n * n * sizeof(double2), c->stream));  // EMPTY
     FS_CUDA(cudaMemsetAsync(D.V.p, 0, (size_t)n * n * sizeof(double2), c->stream));
     {
         int nn = n;
@@ -876,10 +1003,10 @@ void dense_heev(fs_ctx* c, int n, double2* A, int m, double* w, double2* Z, int 
         double* dp = D.d.as<double>();
         double* ep = D.e.as<double>();
         double2* Yp = D.Y.as<double2>();
-        unsigned int* bp = D.bar.as<unsigned int>();
+        double2* Cp = Yp + (size_t)n * n;
         int* errp = ctx_errflag(c);
-        void* args[] = {&nn, &Ap, &Vp, &tp, &dp, &ep, &Yp, &bp, &errp};
-        FS_CUDA(cudaLaunchCooperativeKernel((const void*)hetrd_kernel, nblocks, 256, args, smem, c->stream));
+        void* args[] = {&nn, &Ap, &Vp, &tp, &dp, &ep, &Yp, &Cp, &in_smem, &errp};
+        FS_CUDA(cudaLaunchCooperativeKernel(hk, nblocks, ht, args, smem, c->stream));
     }
     if (n == 1) {
         // no reflector: T = A
@@ -888,32 +1015,42 @@ void dense_heev(fs_ctx* c, int n, double2* A, int m, double* w, double2* Z, int 
     }
     {
     ProfScope ps_t(c, KS_SUB_TRIEIG, 0.0, 0.0);
-    tri_prep_kernel<<<1, 256, 0, c->stream>>>(D.d.as<double>(), D.e.as<double>(), D.e2.as<double>(), n,
-                                              D.info3.as<double>());
-    tri_bisect_kernel<<<m, 32, 0, c->stream>>>(D.d.as<double>(), D.e2.as<double>(), n, m,
-                                                                      D.info3.as<double>(), w);
+    tri_prep_kernel<<<1, 256, 0, c->stream>>>(D.d.as<double>(), D.e.as<double>(), D.ds.as<double>(),
+                                              D.e2.as<double>(), n, D.info3.as<double>());
+    tri_bisect_kernel<<<m, 32, 0, c->stream>>>(D.ds.as<double>(), D.e2.as<double>(), n, m, D.info3.as<double>(), w);
     tri_invit_kernel<<<m, 32, (size_t)8 * n * sizeof(double), c->stream>>>(D.d.as<double>(), D.e.as<double>(), n, m,
-                                                                           w, D.info3.as<double>(), D.z.as<double>());
-    tri_z_to_Z_kernel<<<cdiv((long)n * m, 256), 256, 0, c->stream>>>(n, m, D.z.as<double>(), Z, ldz);
+                                                                           w, D.info3.as<double>(), D.z.as<double>(),
+                                                                           Z, ldz);
     FS_CUDA(cudaGetLastError());
     }
     if (n > 1) {
         ProfScope ps_b(c, KS_SUB_BACK, 0.0, 8.0 * n * (double)n * m);
-        const int nref = n - 1, nblkr = cdiv(nref, NBLK);
-        D.wyT.ensure((size_t)nblkr * NBLK * NBLK * sizeof(double2));
-        D.wyW.ensure((size_t)NBLK * m * sizeof(double2));
-        D.wyW2.ensure((size_t)NBLK * m * sizeof(double2));
+        const int nref = n - 1, nblkr = cdiv(nref, IB);
+        D.wyT.ensure((size_t)nblkr * IB * IB * sizeof(double2));
+        D.linv.ensure((size_t)nblkr * IB * IB * sizeof(double2));
+        D.wyW.ensure((size_t)IB * m * sizeof(double2));
+        D.wyW2.ensure((size_t)IB * m * sizeof(double2));
         double2* W = D.wyW.as<double2>();
         double2* W2 = D.wyW2.as<double2>();
-        const double2* V = D.V.as<double2>();
-        wy_t_kernel<<<nblkr, 256, 0, c->stream>>>(n, V, D.tau.as<double2>(), D.wyT.as<double2>());
-        for (int b = nblkr - 1; b >= 0; --b) {
-            const int j0 = b * NBLK, nbk = std::min(NBLK, nref - j0);
-            const int r0 = j0 + 1, rows = n - r0;  // v_j0 starts at row j0 + 1
+        double2* G = D.wyT.as<double2>();
+        const double2* tau = D.tau.as<double2>();
+        double2* V = D.V.as<double2>();
+        wy_zero_kernel<<<nref, 128, 0, c->stream>>>(n, V, tau);
+        for (int b = 0; b < nblkr; ++b) {
+            const int j0 = b * IB, nbk = std::min(IB, nref - j0), r0 = j0 + 1;  // v_j0 starts at row j0 + 1
             const double2* Vb = V + r0 + (long)j0 * n;
-            const double2* Tb = D.wyT.as<double2>() + (size_t)b * NBLK * NBLK;
+            dense_gemm(c, 1, 0, nbk, nbk, n - r0, 1.0, Vb, n, Vb, n, 0.0, G + (size_t)b * IB * IB, IB);
+            wy_m_kernel<<<cdiv((long)nbk * nbk, 256), 256, 0, c->stream>>>(nbk, G + (size_t)b * IB * IB, tau + j0);
+            tri_inv_kernel<<<IB / 4, 128, 0, c->stream>>>(G + (size_t)b * IB * IB, IB, nbk,
+                                                          D.linv.as<double2>() + (size_t)b * IB * IB);
+        }
+        for (int b = nblkr - 1; b >= 0; --b) {
+            const int j0 = b * IB, nbk = std::min(IB, nref - j0), r0 = j0 + 1, rows = n - r0;
+            const double2* Vb = V + r0 + (long)j0 * n;
+            // T^H = inv(D M') with M' = conj(tau) M of unit diagonal: T^H = inv(M') conj(tau), T = tau inv(M')^H
             dense_gemm(c, 1, 0, nbk, m, rows, 1.0, Vb, n, Z + r0, ldz, 0.0, W, nbk);
-            dense_gemm(c, 0, 0, nbk, m, nbk, 1.0, Tb, nbk, W, nbk, 0.0, W2, nbk);
+            dense_gemm(c, 1, 0, nbk, m, nbk, 1.0, D.linv.as<double2>() + (size_t)b * IB * IB, IB, W, nbk, 0.0, W2, nbk);
+            wy_scale_kernel<<<cdiv((long)nbk * m, 256), 256, 0, c->stream>>>(nbk, m, W2, tau + j0);
             dense_gemm(c, 0, 0, rows, m, nbk, -1.0, Vb, n, W2, nbk, 1.0, Z + r0, ldz);
         }
         FS_CUDA(cudaGetLastError());
@@ -928,13 +1065,15 @@ void dense_heev(fs_ctx* c, int n, double2* A, int m, double* w, double2* Z, int 
         double2* G = D.qrG.as<double2>();
         double2* T = D.qrT.as<double2>();
         dense_gemm(c, 1, 0, m, m, n, 1.0, Z, ldz, Z, ldz, 0.0, G, m);
-        if (dense_potrf(c, m, G, m, nullptr) == 0) {
-            dense_conj_transpose(c, n, m, Z, ldz, T, m);
-            dense_trsm(c, 0, m, n, G, m, T, m);
-            dense_conj_transpose(c, m, n, T, m, Z, ldz);
-        }
+        // (should the factorisation fail, Z stays as it is: decided on the device)
+        D.info.ensure(2 * sizeof(int));
+        int* info = D.info.as<int>() + 1;
+        potrf_async(c, m, G, m, nullptr, info);
+        dense_conj_transpose(c, n, m, Z, ldz, T, m);
+        dense_trsm(c, 0, m, n, G, m, T, m, true);
+        qr_back_kernel<<<cdiv((long)n * m, 256), 256, 0, c->stream>>>(n, m, T, Z, ldz, info);
+        FS_CUDA(cudaGetLastError());
     }
-    ctx_check_errflag(c);
 }
 
 // Generalised Hermitian problem GA x = lambda GB x (both n x n, ld n; GB positive
@@ -948,11 +1087,12 @@ int dense_hegv(fs_ctx* c, int n, double2* GA, double2* GB, int m, double* w) {
     D.T.ensure((size_t)n * n * sizeof(double2));
     D.U.ensure((size_t)n * m * sizeof(double2));
     double2* T = D.T.as<double2>();
-    dense_trsm(c, 0, n, n, GB, n, GA, n);              // L^-1 GA
+    // (dense_heev's own triangular solve replaces the kept inverses)
+    dense_trsm(c, 0, n, n, GB, n, GA, n, true);        // L^-1 GA
     dense_conj_transpose(c, n, n, GA, n, T, n);         // (L^-1 GA)^H = GA L^-H
-    dense_trsm(c, 0, n, n, GB, n, T, n);               // L^-1 GA L^-H
+    dense_trsm(c, 0, n, n, GB, n, T, n, false);        // L^-1 GA L^-H
     dense_heev(c, n, T, m, w, D.U.as<double2>(), n);
-    dense_trsm(c, 1, n, m, GB, n, D.U.as<double2>(), n);  // x = L^-H y
+    dense_trsm(c, 1, n, m, GB, n, D.U.as<double2>(), n, true);  // x = L^-H y
     FS_CUDA(cudaMemcpyAsync(GA, D.U.p, (size_t)n * m * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
     return 0;
 }

@@ -288,7 +288,7 @@ struct Solver {
             ProfScope ps(c, KS_DENSE_LA, 0.0, 8.0 * k * (double)k * k);
             dense_trsm(c, 0, k, k, L, k, C, k);               // L^-1 GA
             dense_conj_transpose(c, k, k, C, k, T, k);          // GA L^-H
-            dense_trsm(c, 0, k, k, L, k, T, k);               // L^-1 GA L^-H
+            dense_trsm(c, 0, k, k, L, k, T, k, false);        // L^-1 GA L^-H
             dense_heev(c, k, T, m, s.evals.as<double>(), C, k);  // m lowest pairs, vectors into C
             dense_trsm(c, 1, k, m, L, k, C, k);               // L^-H V
         }
@@ -798,7 +798,7 @@ fs_status solve_impl(fs_ctx* c, double e_ref, int nstates, double tol, fs_result
         FS_CUDA(cudaMemcpyAsync(c->result_states.as<double2>() + (size_t)i * npw, B64.tX.as<double2>() + (size_t)j * npw,
                                 npw * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
     }
-    FS_CUDA(cudaStreamSynchronize(c->stream));
+    ctx_check_errflag(c);  // (synchronises the stream)
     c->nresult = nstates;
     c->result_eps.assign(res->eps, res->eps + nstates);
     c->result_resid.assign(res->resid, res->resid + nstates);
