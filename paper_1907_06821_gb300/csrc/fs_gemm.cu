@@ -199,19 +199,9 @@ void gemm_gram(fs_ctx* c, int M, int N, int K, const T2* A, long lda, const int*
                  8.0 * M * N * K);
     if constexpr (sizeof(T2) == 16) {
         const bool table = A == c->beta64.as<T2>() && !amap && M == c->nptot && K == c->npw;
-        if (oz_worth(M, N, K)) {
-            oz_gemm(c, M, N, K, OzMat{A, lda, 1, 1, amap}, OzMat{B, ldb, 1, 0, bmap}, OzDst{C, ci, cj}, alpha, beta,
-                    table ? 1 : 0);
-            return;
-        }
-        // FP64 without row maps and with C column-major is a plain GEMM, C = alpha A^H B + beta C
-        // (A, B column-major K x M and K x N): the dense FP64 GEMM (split K when the output is
-        // small), about three times the rate of the row-mapped kernel below
-        if (!amap && !bmap && ci == 1) {
-            dense_gemm(c, 1, 0, M, N, K, alpha, (const double2*)A, (int)lda, (const double2*)B, (int)ldb, beta, C,
-                       (int)cj);
-            return;
-        }
+        dense_gemm_mat(c, M, N, K, alpha, OzMat{A, lda, 1, 1, amap}, OzMat{B, ldb, 1, 0, bmap}, beta, OzDst{C, ci, cj},
+                       table ? 1 : 0, 0);
+        return;
     }
     int tm = (M + BM - 1) / BM, tn = (N + BN - 1) / BN;
     int want = std::max(1, (2 * 152 + tm * tn - 1) / (tm * tn));
@@ -242,17 +232,10 @@ void gemm_nn(fs_ctx* c, int M, int N, int K, const A2* A, long ai, long ak, cons
     ProfScope ps(c, ks_prec<T2>(kid), ((double)K + M * (beta != 0.0 ? 2.0 : 1.0)) * N * sizeof(T2) + (double)M * K * sizeof(A2),
                  8.0 * M * N * K);
     if constexpr (sizeof(T2) == 16 && sizeof(A2) == 16) {
-        if (oz_worth(M, N, K) && (beta == 0.0 || (D == C && ldd == ldc))) {
+        if (beta == 0.0 || (D == C && ldd == ldc)) {
             const bool table = B == c->beta64.as<T2>() && !bmap && N == c->npw && K == c->nptot;
-            oz_gemm(c, N, M, K, OzMat{B, 1, ldb, 0, nullptr, bmap}, OzMat{A, ai, ak, 0},
-                    OzDst{C, 1, ldc, nullptr, cmap}, alpha, beta, table ? 2 : 0);
-            return;
-        }
-        // FP64 without row maps, D aliasing C (or beta = 0) and a unit stride in the coefficients
-        // is a plain GEMM on the column-major views: C (N x M) = B (N x K) op(Acoef) (K x M)
-        if (!bmap && !cmap && (beta == 0.0 || (D == C && ldd == ldc)) && (ak == 1 || ai == 1)) {
-            dense_gemm(c, 0, ak == 1 ? 0 : 2, N, M, K, alpha, (const double2*)B, (int)ldb, (const double2*)A,
-                       (int)(ak == 1 ? ai : ak), beta, (double2*)C, (int)ldc);
+            dense_gemm_mat(c, N, M, K, alpha, OzMat{B, 1, ldb, 0, nullptr, bmap}, OzMat{A, ai, ak, 0}, beta,
+                           OzDst{C, 1, ldc, nullptr, cmap}, table ? 2 : 0, 0);
             return;
         }
     }
