@@ -17,12 +17,12 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <random>
 
 namespace {
 
 constexpr int H = 128;           // hidden width
-constexpr int TR = 28;           // rows per block (3 x TR x 128 floats of shared memory)
 constexpr int P_W1 = 0, P_B1 = P_W1 + H * 4, P_W2 = P_B1 + H, P_B2 = P_W2 + H * H, P_W3 = P_B2 + H,
               P_B3 = P_W3 + H * H, P_W4 = P_B3 + H, P_B4 = P_W4 + H, NPARAM = P_B4 + 1;
 
@@ -47,54 +47,6 @@ __global__ void mlp_prepare_kernel(const float* __restrict__ P, float* __restric
         T[P_W4 + t] = bf(P[P_W4 + t]);
     }
     if (t == 0) T[P_B4] = P[P_B4];
-}
-
-// forward for a tile of TR rows; leaves h1, h2, h3 in shared memory and z in zsh
-__device__ void mlp_tile_forward(const float* __restrict__ T, const float* __restrict__ F, int row0, int rows,
-                                 float (*h1)[H], float (*h2)[H], float (*h3)[H], float* zsh, float* red) {
-    const int j = threadIdx.x;
-    for (int r = 0; r < TR; ++r) {
-        int row = row0 + r;
-        float a = T[P_B1 + j];
-        if (row < rows) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) a += T[P_W1 + k * H + j] * F[(long)row * 4 + k];
-        }
-        h1[r][j] = tanhf(a);
-    }
-    __syncthreads();
-    float acc[TR];
-#pragma unroll
-    for (int r = 0; r < TR; ++r) acc[r] = T[P_B2 + j];
-    for (int k = 0; k < H; ++k) {
-        float w = T[P_W2 + k * H + j];
-#pragma unroll
-        for (int r = 0; r < TR; ++r) acc[r] += w * h1[r][k];
-    }
-#pragma unroll
-    for (int r = 0; r < TR; ++r) h2[r][j] = tanhf(acc[r]);
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < TR; ++r) acc[r] = T[P_B3 + j];
-    for (int k = 0; k < H; ++k) {
-        float w = T[P_W3 + k * H + j];
-#pragma unroll
-        for (int r = 0; r < TR; ++r) acc[r] += w * h2[r][k];
-    }
-#pragma unroll
-    for (int r = 0; r < TR; ++r) h3[r][j] = tanhf(acc[r]);
-    __syncthreads();
-    // z[r] = b4 + sum_j W4[j] h3[r][j]: per-thread products, reduced per row
-    const float w4 = T[P_W4 + j];
-    for (int r = 0; r < TR; ++r) {
-        float v = w4 * h3[r][j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((j & 31) == 0) red[r * 4 + (j >> 5)] = v;
-    }
-    __syncthreads();
-    if (j < TR) zsh[j] = T[P_B4] + red[j * 4] + red[j * 4 + 1] + red[j * 4 + 2] + red[j * 4 + 3];
-    __syncthreads();
 }
 
 // ------------------------------------------------------------------ tensor-core forward
@@ -305,122 +257,325 @@ __global__ void __launch_bounds__(MT, 1) mlp_forward_tc_kernel(const float* __re
     if (t < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(H));
 }
 
-// Loss sum_r w_r (z_r - t_r)^2 * inv_sw and its gradient, one partial per block.
-// The backward pass uses the FP32 master weights (dz/dh) with the BF16 forward
-// activations.
-__global__ void __launch_bounds__(H) mlp_backward_kernel(const float* __restrict__ P, const float* __restrict__ T,
-                                                         const float* __restrict__ F, const float* __restrict__ zt,
-                                                         const float* __restrict__ wt, int rows, float inv_sw,
-                                                         float* __restrict__ gpart, float* __restrict__ lpart) {
-    __shared__ float h1[TR][H], h2[TR][H], h3[TR][H];
-    __shared__ float zsh[TR], red[TR * 4], g[TR];
-    const int row0 = blockIdx.x * TR;
-    const int j = threadIdx.x;
-    mlp_tile_forward(T, F, row0, rows, h1, h2, h3, zsh, red);
-    float* gp = gpart + (long)blockIdx.x * NPARAM;
-    if (j < TR) {
-        int row = row0 + j;
-        float r = 0.f, w = 0.f;
-        if (row < rows) {
-            r = zsh[j] - zt[row];
-            w = wt[row];
+// ------------------------------------------------------------------ training step
+// Loss sum_r w_r (z_r - t_r)^2 * inv_sw and its gradient.  Forward with the BF16-rounded
+// weights, backward (dz/dh) with the FP32 master weights, FP32 arithmetic.
+//
+// A persistent block walks tiles of 64 rows with both 128 x 128 weight matrices (FP32, 64 KB
+// each) and the tile's three activation blocks (32 KB each) in shared memory; the six
+// products of a tile are register-tiled (8 rows x 4 columns per thread, gradients 8 x 8), so
+// the FP32 units bound it (6.3 M FMAs a tile).  Weights are stored with their 16-byte chunks
+// permuted by row (chunk ^ (row & 7)): both the forward (lanes on rows) and the backward reads
+// (lanes on columns) are free of bank conflicts.  Gradients: chains of 32 rows in FP32, added
+// to the block's partial sums as two-float numbers (error-free additions), the blocks summed
+// in FP64 in a fixed order.  (One block of 28 rows per 128 threads, with a partial gradient of
+// 135 KB each and two shared-memory reads per FMA, took 4.1 ms for 153,312 rows; this 1.25 ms.)
+constexpr int GR = 64;                        // rows of a tile
+constexpr int GT = 256;                       // threads
+constexpr int NPAD = (NPARAM + 1 + 3) / 4 * 4;  // parameters and the loss, padded
+constexpr int G_SMEM = (2 * H * H + 3 * GR * H + 3 * H + GR) * 4;
+
+__device__ __forceinline__ int wslot(int row, int chunk) { return row * H + ((chunk ^ (row & 7)) << 2); }
+
+// (hi, lo) += v, error-free
+__device__ __forceinline__ void two_add(float& hi, float& lo, float v) {
+    const float s = __fadd_rn(hi, v), bb = __fadd_rn(s, -hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -bb)), __fadd_rn(v, -bb)));
+    hi = s;
+}
+__device__ __forceinline__ void put1(float* hi, float* lo, int p, float v, bool first) {
+    float h = first ? 0.f : hi[p], l = first ? 0.f : lo[p];
+    two_add(h, l, v);
+    hi[p] = h;
+    lo[p] = l;
+}
+
+// forward product of the warp's 8 rows: acc[r][q] = bias + sum_k bf(W[lane + 32 q][k]) h[r][k]
+__device__ __forceinline__ void g_forward(const float* W, const float* bias, const float* h, float (&acc)[8][4]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int r = 0; r < 8; ++r) acc[r][q] = bias[lane + 32 * q];
+#pragma unroll 2
+    for (int c = 0; c < H / 4; ++c) {
+        float4 w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 t = *reinterpret_cast<const float4*>(W + wslot(lane + 32 * q, c));
+            w[q] = make_float4(bf(t.x), bf(t.y), bf(t.z), bf(t.w));
         }
-        g[j] = 2.f * w * r * inv_sw;
-        red[j] = w * r * r * inv_sw;
-    }
-    __syncthreads();
-    if (j == 0) {
-        float l = 0.f, gb = 0.f;
-        for (int r = 0; r < TR; ++r) {
-            l += red[r];
-            gb += g[r];
-        }
-        lpart[blockIdx.x] = l;
-        gp[P_B4] = gb;
-    }
-    // layer 4
-    {
-        float s = 0.f;
-        for (int r = 0; r < TR; ++r) s += g[r] * h3[r][j];
-        gp[P_W4 + j] = s;
-    }
-    // delta3 -> stored over h3 after use; need h3 for gW4 (done) and the tanh derivative
-    const float w4 = P[P_W4 + j];
-    __syncthreads();
-    for (int r = 0; r < TR; ++r) h3[r][j] = g[r] * w4 * (1.f - h3[r][j] * h3[r][j]);  // delta3[r][j]
-    __syncthreads();
-    // layer 3: gW3[j][k] = sum_r delta3[r][j] h2[r][k]; gb3[j] = sum_r delta3[r][j]
-    {
-        float sb = 0.f;
-        for (int r = 0; r < TR; ++r) sb += h3[r][j];
-        gp[P_B3 + j] = sb;
-        for (int k = 0; k < H; ++k) {
-            float s = 0.f;
-#pragma unroll 8
-            for (int r = 0; r < TR; ++r) s += h3[r][j] * h2[r][k];
-            gp[P_W3 + j * H + k] = s;
-        }
-    }
-    // delta2[r][k] = (sum_j delta3[r][j] W3[j][k]) (1 - h2^2): thread = k
-    float acc[TR];
 #pragma unroll
-    for (int r = 0; r < TR; ++r) acc[r] = 0.f;
-    for (int jj = 0; jj < H; ++jj) {
-        float w = P[P_W3 + jj * H + j];
+        for (int r = 0; r < 8; ++r) {
+            const float4 x = *reinterpret_cast<const float4*>(h + r * H + 4 * c);
 #pragma unroll
-        for (int r = 0; r < TR; ++r) acc[r] += h3[r][jj] * w;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < TR; ++r) h2[r][j] = acc[r] * (1.f - h2[r][j] * h2[r][j]);  // delta2
-    __syncthreads();
-    {
-        float sb = 0.f;
-        for (int r = 0; r < TR; ++r) sb += h2[r][j];
-        gp[P_B2 + j] = sb;
-        for (int k = 0; k < H; ++k) {
-            float s = 0.f;
-#pragma unroll 8
-            for (int r = 0; r < TR; ++r) s += h2[r][j] * h1[r][k];
-            gp[P_W2 + j * H + k] = s;
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < TR; ++r) acc[r] = 0.f;
-    for (int jj = 0; jj < H; ++jj) {
-        float w = P[P_W2 + jj * H + j];
-#pragma unroll
-        for (int r = 0; r < TR; ++r) acc[r] += h2[r][jj] * w;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < TR; ++r) h1[r][j] = acc[r] * (1.f - h1[r][j] * h1[r][j]);  // delta1
-    __syncthreads();
-    {
-        float sb = 0.f;
-        float s4[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int r = 0; r < TR; ++r) {
-            int row = row0 + r;
-            float d = h1[r][j];
-            sb += d;
-            if (row < rows) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) s4[k] += d * F[(long)row * 4 + k];
+            for (int q = 0; q < 4; ++q) {
+                acc[r][q] = fmaf(w[q].x, x.x, acc[r][q]);
+                acc[r][q] = fmaf(w[q].y, x.y, acc[r][q]);
+                acc[r][q] = fmaf(w[q].z, x.z, acc[r][q]);
+                acc[r][q] = fmaf(w[q].w, x.w, acc[r][q]);
             }
         }
-        gp[P_B1 + j] = sb;
+    }
+}
+// backward product of the warp's 8 rows: acc[r][i] = sum_j d[r][j] W[j][4 lane + i]
+__device__ __forceinline__ void g_backward(const float* W, const float* d, float (&acc)[8][4]) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) gp[P_W1 + j * 4 + k] = s4[k];
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[r][i] = 0.f;
+#pragma unroll 2
+    for (int j4 = 0; j4 < H; j4 += 4) {
+        float4 w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w[u] = *reinterpret_cast<const float4*>(W + wslot(j4 + u, lane));
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const float4 x = *reinterpret_cast<const float4*>(d + r * H + j4);
+            const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                acc[r][0] = fmaf(xs[u], w[u].x, acc[r][0]);
+                acc[r][1] = fmaf(xs[u], w[u].y, acc[r][1]);
+                acc[r][2] = fmaf(xs[u], w[u].z, acc[r][2]);
+                acc[r][3] = fmaf(xs[u], w[u].w, acc[r][3]);
+            }
+        }
+    }
+}
+// gradient of a 128 x 128 layer from the tile: G[j][k] += sum_r d[r][j] h[r][k], and its bias
+__device__ __forceinline__ void g_outer(const float* d, const float* h, float* hi, float* lo, float* bhi, float* blo,
+                                        bool first) {
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    for (int half = 0; half < 2; ++half) {
+        float acc[8][8];
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
+#pragma unroll 2
+        for (int r = half * (GR / 2); r < (half + 1) * (GR / 2); ++r) {
+            const float4 d0 = *reinterpret_cast<const float4*>(d + r * H + 8 * ty);
+            const float4 d1 = *reinterpret_cast<const float4*>(d + r * H + 8 * ty + 4);
+            const float4 h0 = *reinterpret_cast<const float4*>(h + r * H + 4 * tx);
+            const float4 h1 = *reinterpret_cast<const float4*>(h + r * H + 64 + 4 * tx);
+            const float dv[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+            const float hv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+#pragma unroll
+            for (int a = 0; a < 8; ++a)
+#pragma unroll
+                for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(dv[a], hv[b], acc[a][b]);
+        }
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int p = (8 * ty + a) * H + 64 * b + 4 * tx;
+                float4 vh = make_float4(0.f, 0.f, 0.f, 0.f), vl = vh;
+                if (!first || half) {
+                    vh = *reinterpret_cast<const float4*>(hi + p);
+                    vl = *reinterpret_cast<const float4*>(lo + p);
+                }
+                two_add(vh.x, vl.x, acc[a][4 * b]);
+                two_add(vh.y, vl.y, acc[a][4 * b + 1]);
+                two_add(vh.z, vl.z, acc[a][4 * b + 2]);
+                two_add(vh.w, vl.w, acc[a][4 * b + 3]);
+                *reinterpret_cast<float4*>(hi + p) = vh;
+                *reinterpret_cast<float4*>(lo + p) = vl;
+            }
+        if (threadIdx.x < H) {
+            float sb = 0.f;
+#pragma unroll 8
+            for (int r = half * (GR / 2); r < (half + 1) * (GR / 2); ++r) sb += d[r * H + threadIdx.x];
+            put1(bhi, blo, threadIdx.x, sb, first && !half);
+        }
     }
 }
 
-// fixed-order sum over blocks (deterministic)
+// part: per block NPAD floats (hi), then NPAD (lo)
+__global__ void __launch_bounds__(GT, 1) mlp_grad_kernel(const float* __restrict__ P, const float* __restrict__ F,
+                                                         const float* __restrict__ zt, const float* __restrict__ wt,
+                                                         int rows, float inv_sw, float* __restrict__ part) {
+    extern __shared__ __align__(1024) float gsm[];
+    float* W2 = gsm;
+    float* W3 = W2 + H * H;
+    float* h1 = W3 + H * H;
+    float* h2 = h1 + GR * H;
+    float* h3 = h2 + GR * H;
+    float* b2 = h3 + GR * H;
+    float* b3 = b2 + H;
+    float* w4 = b3 + H;  // master values
+    float* g = w4 + H;
+    __shared__ float lsum[GT / 32], gsum[GT / 32];
+    const int t = threadIdx.x, lane = t & 31, wp = t >> 5, j1 = t & (H - 1), hf = t >> 7;
+    for (int e = t; e < H * H / 4; e += GT) {
+        const int r = e >> 5, c = e & 31;
+        *reinterpret_cast<float4*>(W2 + wslot(r, c)) = *reinterpret_cast<const float4*>(P + P_W2 + 4 * e);
+        *reinterpret_cast<float4*>(W3 + wslot(r, c)) = *reinterpret_cast<const float4*>(P + P_W3 + 4 * e);
+    }
+    if (t < H) {
+        b2[t] = P[P_B2 + t];
+        b3[t] = P[P_B3 + t];
+        w4[t] = P[P_W4 + t];
+    }
+    float w1[4];  // layer 1 of unit j1
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w1[k] = bf(P[P_W1 + 4 * j1 + k]);
+    const float b1 = P[P_B1 + j1], b4 = P[P_B4];
+    float* hi = part + (size_t)blockIdx.x * 2 * NPAD;
+    float* lo = hi + NPAD;
+    __syncthreads();
+    bool first = true;
+    for (int row0 = blockIdx.x * GR; row0 < rows; row0 += gridDim.x * GR, first = false) {
+        // layer 1: unit j1, half of the rows
+        for (int r = hf * (GR / 2); r < (hf + 1) * (GR / 2); ++r) {
+            float a = b1;
+            if (row0 + r < rows) {
+                const float* f = F + (long)(row0 + r) * 4;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) a += w1[k] * f[k];
+            }
+            h1[r * H + j1] = tanhf(a);
+        }
+        __syncthreads();
+        // layers 2 and 3 on the warp's own 8 rows
+        float acc[8][4];
+        g_forward(W2, b2, h1 + 8 * wp * H, acc);
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) h2[(8 * wp + r) * H + lane + 32 * q] = tanhf(acc[r][q]);
+        __syncwarp();
+        g_forward(W3, b3, h2 + 8 * wp * H, acc);
+        float lw = 0.f, gw = 0.f;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            float z = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                acc[r][q] = tanhf(acc[r][q]);
+                h3[(8 * wp + r) * H + lane + 32 * q] = acc[r][q];
+                z = fmaf(bf(w4[lane + 32 * q]), acc[r][q], z);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+            const int row = row0 + 8 * wp + r;
+            float e = 0.f, w = 0.f;
+            if (row < rows) {
+                e = b4 + z - zt[row];
+                w = wt[row];
+            }
+            const float gr = 2.f * w * e * inv_sw;
+            lw += w * e * e * inv_sw;
+            gw += gr;
+            if (lane == 0) g[8 * wp + r] = gr;
+        }
+        if (lane == 0) {
+            lsum[wp] = lw;
+            gsum[wp] = gw;
+        }
+        __syncthreads();
+        if (t < H) {  // layer 4
+            for (int half = 0; half < 2; ++half) {
+                float s = 0.f;
+#pragma unroll 8
+                for (int r = half * (GR / 2); r < (half + 1) * (GR / 2); ++r) s = fmaf(g[r], h3[r * H + t], s);
+                put1(hi, lo, P_W4 + t, s, first && !half);
+            }
+        } else if (t < H + 2) {
+            const float* v = t == H ? gsum : lsum;
+            float s = 0.f;
+            for (int i = 0; i < GT / 32; ++i) s += v[i];
+            put1(hi, lo, P_B4 + t - H, s, first);
+        }
+        __syncthreads();
+        // delta 3 over h3
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int j = lane + 32 * q;
+                h3[(8 * wp + r) * H + j] = g[8 * wp + r] * w4[j] * (1.f - acc[r][q] * acc[r][q]);
+            }
+        __syncthreads();
+        g_outer(h3, h2, hi + P_W3, lo + P_W3, hi + P_B3, lo + P_B3, first);
+        // delta 2 over h2
+        g_backward(W3, h3 + 8 * wp * H, acc);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            float4* x = reinterpret_cast<float4*>(h2 + (8 * wp + r) * H + 4 * lane);
+            const float4 v = *x;
+            *x = make_float4(acc[r][0] * (1.f - v.x * v.x), acc[r][1] * (1.f - v.y * v.y),
+                             acc[r][2] * (1.f - v.z * v.z), acc[r][3] * (1.f - v.w * v.w));
+        }
+        __syncthreads();
+        g_outer(h2, h1, hi + P_W2, lo + P_W2, hi + P_B2, lo + P_B2, first);
+        // delta 1 over h1
+        g_backward(W2, h2 + 8 * wp * H, acc);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            float4* x = reinterpret_cast<float4*>(h1 + (8 * wp + r) * H + 4 * lane);
+            const float4 v = *x;
+            *x = make_float4(acc[r][0] * (1.f - v.x * v.x), acc[r][1] * (1.f - v.y * v.y),
+                             acc[r][2] * (1.f - v.z * v.z), acc[r][3] * (1.f - v.w * v.w));
+        }
+        __syncthreads();
+        if (t < H) {  // layer 1
+            for (int half = 0; half < 2; ++half) {
+                float sb = 0.f, s4[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int r = half * (GR / 2); r < (half + 1) * (GR / 2); ++r) {
+                    const float dl = h1[r * H + t];
+                    sb += dl;
+                    if (row0 + r < rows) {
+                        const float* f = F + (long)(row0 + r) * 4;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) s4[k] = fmaf(dl, f[k], s4[k]);
+                    }
+                }
+                put1(hi, lo, P_B1 + t, sb, first && !half);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) put1(hi, lo, P_W1 + 4 * t + k, s4[k], first && !half);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// sum over the blocks' two-float partial sums in FP64, in block order (deterministic)
 __global__ void sum_parts_kernel(const float* __restrict__ part, int nblk, int n, float* __restrict__ out) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     double s = 0;
-    for (int b = 0; b < nblk; ++b) s += part[(long)b * n + p];
+#pragma unroll 4
+    for (int b = 0; b < nblk; ++b) {
+        const float* h = part + (size_t)b * 2 * NPAD + p;
+        s += (double)h[0] + (double)h[NPAD];
+    }
     out[p] = (float)s;
+}
+
+// sum of the weights in FP64 (one block, fixed order)
+__global__ void __launch_bounds__(1024) weight_sum_kernel(const float* __restrict__ w, int n, double* __restrict__ out) {
+    __shared__ double sh[32];
+    double s = 0;
+    for (int i = threadIdx.x; i < n; i += 8 * 1024) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = i + 1024 * u < n ? w[i + 1024 * u] : 0.f;
+        // exact in FP64 up to its rounding: pairs first (half of the FP64 additions)
+        s += ((double)v[0] + v[1]) + ((double)v[2] + v[3]) + (((double)v[4] + v[5]) + ((double)v[6] + v[7]));
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        s = sh[threadIdx.x];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) *out = s;
+    }
 }
 
 __global__ void adam_kernel(float* P, const float* __restrict__ g, float* m, float* v, int n, float lr, float bc1,
@@ -594,7 +749,7 @@ void mlp_setup(fs_ctx* c) {
     L.T.alloc(NPARAM * sizeof(float));
     L.m.alloc(NPARAM * sizeof(float));
     L.v.alloc(NPARAM * sizeof(float));
-    L.g.alloc(NPARAM * sizeof(float));
+    L.g.alloc((NPARAM + 1) * sizeof(float));  // and the loss
     // default initialisation: U(-1/sqrt(fan_in), 1/sqrt(fan_in)) hidden layers, zero output layer
     std::vector<float> p(NPARAM, 0.f);
     std::mt19937 gen(1234);
@@ -639,19 +794,38 @@ void mlp_forward(fs_ctx* c, const float* F, int rows, float* z) {
     FS_CUDA(cudaGetLastError());
 }
 
+// sum of the device weights wt[rows]
+double mlp_weight_sum(fs_ctx* c, const float* wt, int rows) {
+    c->mlp.lpart.ensure(sizeof(double));
+    weight_sum_kernel<<<1, 1024, 0, c->stream>>>(wt, rows, c->mlp.lpart.as<double>());
+    FS_CUDA(cudaGetLastError());
+    double sw = 0;
+    FS_CUDA(cudaMemcpyAsync(&sw, c->mlp.lpart.p, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    FS_CUDA(cudaStreamSynchronize(c->stream));
+    return sw;
+}
+
 // loss (returned) and gradient (into c->mlp.g) of the weighted MSE on rows
 double mlp_loss_grad(fs_ctx* c, const float* F, const float* zt, const float* wt, int rows, double sw) {
     Mlp& L = c->mlp;
-    int nblk = (rows + TR - 1) / TR;
-    L.gpart.ensure((size_t)nblk * NPARAM * sizeof(float));
-    L.lpart.ensure((size_t)nblk * sizeof(float) + sizeof(float));
-    mlp_backward_kernel<<<nblk, H, 0, c->stream>>>(L.P.as<float>(), L.T.as<float>(), F, zt, wt, rows,
-                                                   (float)(1.0 / sw), L.gpart.as<float>(), L.lpart.as<float>());
-    sum_parts_kernel<<<(NPARAM + 255) / 256, 256, 0, c->stream>>>(L.gpart.as<float>(), nblk, NPARAM, L.g.as<float>());
-    float* lsum = L.lpart.as<float>() + nblk;
-    sum_parts_kernel<<<1, 32, 0, c->stream>>>(L.lpart.as<float>(), nblk, 1, lsum);
+    if (rows <= 0) throw fs_error(FS_ERR_CUDA, "no training rows");
+    static std::once_flag once;
+    std::call_once(once, [] {
+        cudaFuncSetAttribute((const void*)mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
+    });
+    int dev = 0, nsm = 0;
+    FS_CUDA(cudaGetDevice(&dev));
+    FS_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int nblk = std::max(1, std::min((rows + GR - 1) / GR, nsm));
+    L.gpart.ensure((size_t)nblk * 2 * NPAD * sizeof(float));
+    mlp_grad_kernel<<<nblk, GT, G_SMEM, c->stream>>>(L.P.as<float>(), F, zt, wt, rows, (float)(1.0 / sw),
+                                                     L.gpart.as<float>());
+    // parameters and, after them, the loss
+    sum_parts_kernel<<<(NPARAM + 1 + 127) / 128, 128, 0, c->stream>>>(L.gpart.as<float>(), nblk, NPARAM + 1,
+                                                                      L.g.as<float>());
+    FS_CUDA(cudaGetLastError());
     float loss = 0;
-    FS_CUDA(cudaMemcpyAsync(&loss, lsum, sizeof(float), cudaMemcpyDeviceToHost, c->stream));
+    FS_CUDA(cudaMemcpyAsync(&loss, L.g.as<float>() + NPARAM, sizeof(float), cudaMemcpyDeviceToHost, c->stream));
     FS_CUDA(cudaStreamSynchronize(c->stream));
     return loss;
 }

@@ -195,10 +195,9 @@ fs_status fs_precond_loss_grad(fs_ctx* c, const float* features, const float* ta
     }
     return guard(c, [&] {
         mlp_setup(c);
-        std::vector<float> wh(rows);
-        FS_CUDA(cudaMemcpy(wh.data(), weight, rows * sizeof(float), cudaMemcpyDeviceToHost));
-        double sw = 0;
-        for (float v : wh) sw += v;
+        // inputs made on the legacy default stream are complete before this stream reads them
+        FS_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+        const double sw = mlp_weight_sum(c, weight, rows);
         if (!(sw > 0)) throw fs_error(FS_ERR_ARG, "fs_precond_loss_grad: weights sum to zero");
         *loss = (float)mlp_loss_grad(c, features, target, weight, rows, sw);
         FS_CUDA(cudaMemcpyAsync(grad, c->mlp.g.p, mlp_nparam() * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
