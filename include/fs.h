@@ -94,7 +94,7 @@ typedef struct {
     unsigned long long seed;   /* start block when none is supplied */
     void* cuda_stream;         /* cudaStream_t to run on (NULL: the library's own stream) */
     int verbose;               /* > 0: one line per iteration on stderr */
-    int gemm_path;             /* FP32-stage GEMMs: FS_GEMM_TENSOR (default, tcgen05 TF32 x3 split)
+    int gemm_path;             /* FP32-stage GEMMs: FS_GEMM_TENSOR (default, tcgen05, FP16 x3 split)
                                   or FS_GEMM_CUDA_CORES (FP32 FMA); FP64 work always uses FP64 FMA */
     int projectors;            /* FS_PROJ_AUTO (0, default): the projector table beta[N_p][npw] is
                                   stored when its FP64 form takes at most 16 GB, else generated;

@@ -205,15 +205,14 @@ void ensure_fp32_tables(fs_ctx* c) {
 
 void ctx_ensure_fp32(fs_ctx* c) { ensure_fp32_tables(c); }
 
-int* ctx_errflag(fs_ctx* c) { return c->errflag.as<int>(); }
+int* ctx_errflag(fs_ctx* c) { return c->errflag_dev; }
 
-// raise FS_ERR_TIMEOUT if a device-side bounded wait gave up (clears the flag)
+// wait for the stream and raise FS_ERR_TIMEOUT if a device-side bounded wait gave up (clears
+// the flag, which lives in mapped host memory: reading it costs no copy)
 void ctx_check_errflag(fs_ctx* c) {
-    int v = 0;
-    FS_CUDA(cudaMemcpyAsync(&v, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     FS_CUDA(cudaStreamSynchronize(c->stream));
-    if (v) {
-        FS_CUDA(cudaMemsetAsync(c->errflag.p, 0, sizeof(int), c->stream));
+    if (*(volatile int*)c->errflag) {
+        *(volatile int*)c->errflag = 0;
         throw fs_error(FS_ERR_TIMEOUT, "a tensor-core pipeline wait exceeded its limit");
     }
 }
@@ -248,8 +247,9 @@ fs_status fs_create(const fs_grid* grid, double ecut, const double k[3], const d
             throw fs_error(FS_ERR_ARG, "bad gemm_path");
         c->gemm_path = c->opt.gemm_path;
         FS_CUDA(cudaGetDevice(&c->device));
-        c->errflag.alloc(sizeof(int));
-        FS_CUDA(cudaMemset(c->errflag.p, 0, sizeof(int)));
+        FS_CUDA(cudaHostAlloc((void**)&c->errflag, sizeof(int), cudaHostAllocMapped));
+        *c->errflag = 0;
+        FS_CUDA(cudaHostGetDevicePointer((void**)&c->errflag_dev, c->errflag, 0));
         if (c->opt.cuda_stream) {
             c->stream = (cudaStream_t)c->opt.cuda_stream;
         } else {
@@ -301,8 +301,7 @@ fs_status fs_apply_H(fs_ctx* c, const void* psi, void* hpsi, int nband, double s
             ensure_fp32_tables(c);
             apply_H_impl<float2>(c, (const float2*)psi, (float2*)hpsi, nband, shift);
         }
-        FS_CUDA(cudaStreamSynchronize(c->stream));
-        ctx_check_errflag(c);
+        ctx_check_errflag(c);  // (waits for the stream)
     });
 }
 
@@ -367,6 +366,7 @@ void fs_destroy(fs_ctx* c) {
     prof_release(c);
     cudaStream_t s = c->stream;
     bool own = c->own_stream;
+    if (c->errflag) cudaFreeHost(c->errflag);
     delete c;
     if (own && s) cudaStreamDestroy(s);
 }

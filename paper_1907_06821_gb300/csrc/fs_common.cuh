@@ -285,12 +285,11 @@ struct fs_ctx {
     dbuf projbuf;     // [nb][nptot] complex (P)
     dbuf projbuf2;    // [nb][nptot] complex (Q = D P)
     dbuf splitk;      // split-K partial sums
-    dbuf beta32_fmt;  // projector table as tensor-core apply-form operand images (formatted once)
-    dbuf afmt;        // apply-form operand images of a band block (per call)
-    dbuf bfmt;        // apply-form coefficient images (per call)
-    dbuf beta32_gfmt; // projector table as Gram-form operand images (formatted once)
-    dbuf gfmt_a;      // Gram-form images of the first operand (per call)
-    dbuf gfmt_b;      // Gram-form images of the second operand with rotated rows (per call)
+    dbuf beta32_fmt;  // projector table as tensor-core operand images, rows = plane waves (formatted once)
+    dbuf beta32_gfmt; // the same, rows = projectors
+    dbuf afmt, bfmt;  // operand images of a call
+    dbuf tc_gmax, tc_nmax;  // row maxima of the two table images
+    dbuf tc_ma, tc_mb;      // row maxima of a call's operands
 
     // solver state
     dbuf init_states; // double2 [ninit][npw]
@@ -313,7 +312,8 @@ struct fs_ctx {
     DenseWork dense;
     OzWork oz;
     SolverMem smem;
-    dbuf errflag;     // int: set by a device-side wait that gave up
+    int* errflag = nullptr;      // set by a device-side wait that gave up (mapped host memory)
+    int* errflag_dev = nullptr;  // its device address
     int gemm_path = 0;
     std::string err;
 };

@@ -476,7 +476,7 @@ hetrd_kernel(int n, double2* A, double2* V, double2* tau, double* d, double* e, 
 #pragma unroll
                 for (int q = 0; q < PER; ++q) more = more || is_empty(y[q]) || is_empty(c[q]);
                 if (more && (++it > BAR_LIMIT || ((it & 1023) == 0 && *(volatile int*)err))) {
-                    atomicExch(err, 1);
+                    *(volatile int*)err = 1;
                     gave_up = 1;
                     break;
                 }

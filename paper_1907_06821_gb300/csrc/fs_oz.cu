@@ -431,7 +431,7 @@ oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const un
                 }
         }
     }
-    if (!ok) atomicExch(errflag, 1);
+    if (!ok) *(volatile int*)errflag = 1;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));

@@ -15,7 +15,7 @@
 //   X <- S c (lowest m), P <- [W P] c_WP; Y, YP by linearity.
 // Convergence: a Rayleigh-Ritz step on H within the wanted bands; their H
 // residuals must be <= tol for the nstates pairs nearest E.
-// Mixed precision: vectors, FFTs and GEMMs in FP32 (tensor-core TF32 x3),
+// Mixed precision: vectors, FFTs and GEMMs in FP32 (tensor cores, two-part FP16 split),
 // dense algebra in FP64, Y (and YP) recomputed every 10 iterations; then an
 // FP64 check of the wanted bands, and FP64 iterations only if it fails.
 //
