@@ -21,10 +21,11 @@
 // Why: GB300 does about 2 FP64 FMAs per clock and SM (0.65 TFLOP/s through a GEMM);
 // 34 BF16 digit products at the tensor rate are some 50 times as fast.  What bounds
 // it then: with few columns the digit images (28 bytes per complex element) from
-// HBM; with many the shared-memory reads of the MMAs (M = 128, N <= 64).  Measured:
-// 272 x 272 x 193,673 in 8.6 ms (13 TFLOP/s) against about 180 ms, relative error
-// 1.4e-16 against 0.5 to 1.2e-15; an FP64 H application of 16 bands of 193,673 plane
-// waves with 2,048 projectors (table image kept) in 8.8 ms against 305 ms.
+// HBM; with many the MMAs and the formatting passes.  Measured: 272 x 272 x 193,673 in
+// 7.6 ms (15 TFLOP/s, formatting included) against about 180 ms, relative error 1.4e-16
+// against 0.5 to 1.2e-15; an FP64 H application of 16 bands of 193,673 plane waves with
+// 2,048 projectors (table images kept) in 6.7 ms against 305 ms, 2.1 ms for each of its
+// two products (11 GB of digits: 1.6 ms).
 //
 // Layout.  The complex product is carried by interleaved real rows: the A image of a
 // row holds (re, im) pairs, the B image two rows per n, (re, -im) and (im, re) of b
@@ -260,8 +261,8 @@ struct OzOut {
     double2* part;     // split K: partial (z, n, m) at part[(z * N + n) * M + m] (raw sums), else null
 };
 
-// grid (jtiles, itiles, splits).  Warp 0 copies the stages, warp 1 issues the 34 MMAs
-// of each (digit pairs i + j <= 7 into accumulator i + j), warps 2-9 drain the eight
+// grid (jtiles, itiles, splits).  Warp 0 copies the stages, warp 1 issues the MMAs of
+// each (34 digit pairs i + j <= 7 into accumulator i + j), warps 2-9 drain the eight
 // accumulators of a chain (thread: row 32 (warp & 3) + lane, half of the columns).
 // Two accumulator sets when 16 N2 <= 512 columns of tensor memory, else one.
 __global__ void __launch_bounds__(O_THREADS, 1)
@@ -324,8 +325,9 @@ oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const un
     } else if (warp == 1) {
         if (lane == 0) {
             // kind::f16, BF16 A and B, FP32 D, K-major both
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N2 >> 3) << 17) |
-                                   ((uint32_t)(OM >> 4) << 24);
+            // (the number of columns is added per MMA)
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(OM >> 4) << 24);
+            const int per = 256 / N2;  // digits of B per MMA
             int last = -1;
             for (int kb = 0; kb < nk; ++kb) {
                 const int s = kb % nst, ch = kb / OCHAIN, buf = ch % nbuf;
@@ -342,13 +344,23 @@ oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const un
                 const uint32_t base = oz_smem(smem + (size_t)s * sbytes);
                 const uint64_t ad = oz_desc(base), bd = oz_desc(base + OA_STAGE);
                 const uint32_t d0 = tmem + (uint32_t)(buf * ND * N2);
+                // digit i of A times digits j0 .. j1 of B at once: the slices of B follow one
+                // another in shared memory as the accumulators i + j do in tensor memory, so
+                // they are one operand of (j1 - j0) N2 <= 256 rows.  (One MMA per pair read A
+                // from shared memory 34 times a stage and ran below the full rate at N <= 64.)
 #pragma unroll
-                for (int i = 0; i < NS; ++i)
-#pragma unroll
-                    for (int j = 0; j < (i == 0 ? NS : ND - i); ++j)
-                        oz_mma(d0 + (uint32_t)((i + j) * N2), ad + (uint64_t)((i * OA_SLICE) >> 4),
-                               bd + (uint64_t)((j * bslice) >> 4), idesc,
-                               (first && (i == 0 || (i == 1 && j == NS - 1))) ? 0u : 1u);
+                for (int i = 0; i < NS; ++i) {
+                    const int nj = i == 0 ? NS : ND - i;
+                    for (int j0 = 0, j1; j0 < nj; j0 = j1) {
+                        j1 = min(nj, j0 + per);
+                        // accumulator 7 starts with (1, 6), the others with i = 0
+                        if (first && i == 1 && j0 < NS - 1) j1 = min(j1, NS - 1);
+                        const uint32_t acc = first && (i == 0 || (i == 1 && j0 == NS - 1)) ? 0u : 1u;
+                        oz_mma(d0 + (uint32_t)((i + j0) * N2), ad + (uint64_t)((i * OA_SLICE) >> 4),
+                               bd + (uint64_t)((j0 * bslice) >> 4), idesc + ((uint32_t)((j1 - j0) * (N2 >> 3)) << 17),
+                               acc);
+                    }
+                }
                 oz_commit(&empty[s]);
                 if (kb % OCHAIN == OCHAIN - 1 || kb == nk - 1) oz_commit(&accf[buf]);
                 last = kb;
