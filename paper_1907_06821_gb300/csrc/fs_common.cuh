@@ -216,7 +216,7 @@ struct OzWork {
 };
 
 struct SolverSmall {
-    dbuf GA, GB, T1, T2, evals, work, info, theta, act, resid, dots, nrm, shift, dscale, bkin, hres, keep;
+    dbuf GA, GB, T1, T2, evals, work, info, theta, act, resid, dots, nrm, shift, dscale, bkin, hres, keep, rows;
     int lwork = 0;
     int nbmax = 0;
 };
@@ -354,6 +354,16 @@ template <typename T2, typename A2>
 void gemm_nn(fs_ctx* c, int M, int N, int K, const A2* A, long ai, long ak, const T2* B, long ldb, const int* bmap,
              T2* C, long ldc, const int* cmap, double alpha, double beta, const T2* D, long ldd, int kid = KS_ROTATE);
 
+// the same with rows given by device pointers (several blocks of a basis at once):
+// gemm_gram_rows: C(i, j) = sum_k conj(A[i][k]) B[j][k], both n rows, C column-major (ld n); with
+//   lower only the tiles that reach the lower triangle are computed (C Hermitian)
+// gemm_nn_rows  : C[i][g] = sum_k A(i, k) B[k][g], B's K rows by pointers
+// false where only the CUDA-core FP32 kernels may be used (nothing done)
+template <typename T2>
+bool gemm_gram_rows(fs_ctx* c, int n, int K, const T2* const* A, const T2* const* B, double2* C, int lower);
+template <typename T2>
+bool gemm_nn_rows(fs_ctx* c, int M, int N, int K, const double2* A, long ai, const T2* const* B, T2* C, long ldc);
+
 // tensor-core GEMMs for the FP32 stage (fs_tc.cu); gen: the table operand (A of the
 // Gram form, B of the apply form) is the generated projector table (fs_beta.cuh)
 struct BetaGen;
@@ -364,6 +374,9 @@ template <typename A2>
 void tc_gemm_nn(fs_ctx* c, int M, int N, int K, const A2* A, long ai, long ak, const float2* B, long ldb,
                 const int* bmap, float2* C, long ldc, const int* cmap, double alpha, double beta, const float2* D,
                 long ldd, int kid, const BetaGen* gen = nullptr);
+void tc_gemm_gram_rows(fs_ctx* c, int n, int K, const float2* const* A, const float2* const* B, double2* C, int lower);
+void tc_gemm_nn_rows(fs_ctx* c, int M, int N, int K, const double2* A, long ai, const float2* const* B, float2* C,
+                     long ldc);
 // generated projectors (fs_beta.cu)
 void beta_gen_setup(fs_ctx* c, const fs_projectors* pr, double omega);
 template <typename T2> void beta_project_chunked(fs_ctx* c, const T2* psi, const int* rowmap, int nb, double2* P);
@@ -372,17 +385,16 @@ int* ctx_errflag(fs_ctx* c);
 void ctx_check_errflag(fs_ctx* c);
 
 // vector kernels (fs_vec.cu)
-template <typename T2> void vec_resid(fs_ctx* c, const T2* X, const T2* Y, int m, double* resid, double2* dot);
+template <typename T2>
+void vec_resid(fs_ctx* c, const T2* X, const T2* Y, int m, double* resid, double2* dot, T2* RH);
 template <typename T2>
 void vec_make_w(fs_ctx* c, const T2* R, const int* act, int na, T2* W, double e_ref, double dE, int precond,
                 const double* band_kin);
-template <typename T2> void vec_rh(fs_ctx* c, const T2* X, const T2* Y, const double2* dots, int m, T2* RH);
 template <typename T2>
 void vec_a_resid(fs_ctx* c, const T2* ZR, T2* RH, const T2* X, const double2* dots, const double* theta, int m,
                  double* ra);
-template <typename T2> void vec_row_norms(fs_ctx* c, const T2* X, const int* map, int nrows, double* out);
+template <typename T2> void vec_normalize(fs_ctx* c, T2* X, T2* Y, const int* map, int nrows);
 template <typename T2> void vec_band_kin(fs_ctx* c, const T2* X, int m, double* out);
-template <typename T2> void vec_scale_rows(fs_ctx* c, T2* X, const int* map, int nrows, const double* nrm);
 template <typename T2>
 void vec_resid_shift(fs_ctx* c, const T2* X, const T2* Y, const double* shift, int m, double* resid);
 void vec_damp_random(fs_ctx* c, double2* X, int m, int first, unsigned long long seed);
@@ -412,6 +424,8 @@ struct OzMat {
     long sr, sk;
     int conj;
     const int *map = nullptr, *kmap = nullptr;
+    const double2* const* rp = nullptr;
+    const double2* const* kp = nullptr;
 };
 struct OzDst {
     double2* C;

@@ -56,6 +56,8 @@ __device__ __forceinline__ double2 zconj(double2 a) { return make_double2(a.x, -
 // lower = 1: tiles wholly above the diagonal (every row index below every column
 // index) are skipped, for updates of which only the lower triangle is used.
 __device__ __forceinline__ const double2* mat_at(const OzMat& A, int r, int k) {
+    if (A.rp) return A.rp[r] + (long)k * A.sk;
+    if (A.kp) return A.kp[k] + (long)r * A.sr;
     return A.X + (A.map ? (long)A.map[r] : (long)r) * A.sr + (A.kmap ? (long)A.kmap[k] : (long)k) * A.sk;
 }
 
@@ -790,15 +792,24 @@ __global__ void wy_scale_kernel(int b, int m, double2* X, const double2* tau) {
 
 inline int cdiv(long a, long b) { return (int)((a + b - 1) / b); }
 
-// C(m, n) = alpha sum_z P(z, n, m) + beta C(m, n), z in order
-__global__ void gemm_sum_kernel(int M, int N, int splits, const double2* P, double alpha, double beta, OzDst C,
-                                int lower) {
-    long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (t >= (long)M * N) return;
+// C(m, n) = alpha sum_z P(z, n, m) + beta C(m, n): 32 outputs per block, eight groups of
+// consecutive z added in order (deterministic)
+__global__ void __launch_bounds__(256) gemm_sum_kernel(int M, int N, int splits, const double2* P, double alpha,
+                                                       double beta, OzDst C, int lower) {
+    __shared__ double2 sh[8][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long total = (long)M * N, t = blockIdx.x * 32l + lane;
     const int m = (int)(t % M), n = (int)(t / M);
-    if (lower && (m / TB + 1) * TB <= (n / TB) * TB) return;  // a tile the GEMM skipped
-    double2 s = P[t];
-    for (int z = 1; z < splits; ++z) s = cadd(s, P[(size_t)z * M * N + t]);
+    const bool live = t < total && !(lower && (m / TB + 1) * TB <= (n / TB) * TB);  // (a tile the GEMM skipped)
+    const int per = (splits + 7) / 8, z1 = min(splits, (w + 1) * per);
+    double2 s = make_double2(0.0, 0.0);
+    if (live)
+#pragma unroll 4
+        for (int z = w * per; z < z1; ++z) s = cadd(s, P[(size_t)z * total + t]);
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w || !live) return;
+    for (int i = 1; i < 8; ++i) s = cadd(s, sh[i][lane]);
     double2* c = C.C + (C.mmap ? (long)C.mmap[m] : (long)m) * C.cm + (C.nmap ? (long)C.nmap[n] : (long)n) * C.cn;
     double2 o = make_double2(alpha * s.x, alpha * s.y);
     if (beta != 0.0) {
@@ -840,13 +851,15 @@ void dense_gemm_mat(fs_ctx* c, int M, int N, int K, double alpha, const OzMat& A
         OzDst d = C;
         const int ny = std::min(N - y0, 65535 * TB);
         if (y0) {
-            if (b.map) b.map += y0; else b.X += (long)y0 * b.sr;
+            if (b.rp) b.rp += y0;
+            else if (b.map) b.map += y0;
+            else b.X += (long)y0 * b.sr;
             if (d.nmap) d.nmap += y0; else d.C += (long)y0 * d.cn;
         }
         zgemm_kernel<<<dim3(cdiv(M, TB), cdiv(ny, TB), splits), TB * TB, 0, c->stream>>>(M, ny, K, alpha, A, b, beta, d,
                                                                                       P, kc, lower);
         if (P)
-            gemm_sum_kernel<<<cdiv((long)M * ny, 256), 256, 0, c->stream>>>(M, ny, splits, P, alpha, beta, d, lower);
+            gemm_sum_kernel<<<cdiv((long)M * ny, 32), 256, 0, c->stream>>>(M, ny, splits, P, alpha, beta, d, lower);
     }
     FS_CUDA(cudaGetLastError());
 }

@@ -256,6 +256,41 @@ template void gemm_nn<float2, double2>(fs_ctx*, int, int, int, const double2*, l
                                        const int*, float2*, long, const int*, double, double, const float2*, long,
                                        int);
 
+template <typename T2>
+bool gemm_gram_rows(fs_ctx* c, int n, int K, const T2* const* A, const T2* const* B, double2* C, int lower) {
+    if constexpr (sizeof(T2) == 8) {
+        if (c->gemm_path != FS_GEMM_TENSOR) return false;
+        tc_gemm_gram_rows(c, n, K, A, B, C, lower);
+    } else {
+        ProfScope ps(c, KS_GRAM64, 2.0 * n * K * sizeof(T2), 8.0 * n * (double)n * K);
+        OzMat a{nullptr, 0, 1, 1}, b{nullptr, 0, 1, 0};
+        a.rp = A;
+        b.rp = B;
+        // (the tensor-core form computes every tile)
+        dense_gemm_mat(c, n, n, K, 1.0, a, b, 0.0, OzDst{C, 1, n}, 0, lower && !oz_worth(n, n, K));
+    }
+    return true;
+}
+
+template <typename T2>
+bool gemm_nn_rows(fs_ctx* c, int M, int N, int K, const double2* A, long ai, const T2* const* B, T2* C, long ldc) {
+    if constexpr (sizeof(T2) == 8) {
+        if (c->gemm_path != FS_GEMM_TENSOR) return false;
+        tc_gemm_nn_rows(c, M, N, K, A, ai, B, C, ldc);
+    } else {
+        ProfScope ps(c, KS_ROTATE64, ((double)K + M) * N * sizeof(T2), 8.0 * M * (double)N * K);
+        OzMat b{nullptr, 1, 0, 0};
+        b.kp = B;
+        dense_gemm_mat(c, N, M, K, 1.0, b, OzMat{A, ai, 1, 0}, 0.0, OzDst{C, 1, ldc}, 0, 0);
+    }
+    return true;
+}
+template bool gemm_gram_rows<float2>(fs_ctx*, int, int, const float2* const*, const float2* const*, double2*, int);
+template bool gemm_gram_rows<double2>(fs_ctx*, int, int, const double2* const*, const double2* const*, double2*, int);
+template bool gemm_nn_rows<float2>(fs_ctx*, int, int, int, const double2*, long, const float2* const*, float2*, long);
+template bool gemm_nn_rows<double2>(fs_ctx*, int, int, int, const double2*, long, const double2* const*, double2*,
+                                    long);
+
 // Gram form with caller-provided split-K scratch (no allocation): the same
 // kernels as gemm_gram on CUDA cores; part must hold splits * M * N double2.
 // Returns false when the scratch is too small for even one split.

@@ -133,6 +133,13 @@ struct OzOp {
     long sr, sk;
     const int* map;
     const int* kmap;
+    const double2* const* rp;  // rows, or k, by pointers
+    const double2* const* kp;
+    __device__ __forceinline__ const double2& at(int r, long k) const {
+        if (rp) return rp[r][k * sk];
+        if (kp) return kp[k][r * sr];
+        return X[(map ? (long)map[r] : (long)r) * sr + (kmap ? (long)kmap[k] : k) * sk];
+    }
 };
 
 // largest magnitude (as bits) of every row over k in [0, K).  sk = 1: a warp walks along k;
@@ -142,10 +149,10 @@ __global__ void oz_max_kernel(OzOp op, int R, int K, int kper, unsigned long lon
     if (op.sk == 1) {
         const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
         if (r >= R) return;
-        const double2* x = op.X + (op.map ? (long)op.map[r] : (long)r) * op.sr;
         unsigned long long m = 0;
+#pragma unroll 4
         for (int k = k0 + lane; k < k1; k += 32) {
-            const double2 v = x[op.kmap ? op.kmap[k] : k];
+            const double2 v = op.at(r, k);
             m = max(m, max((unsigned long long)__double_as_longlong(v.x) & 0x7fffffffffffffffull,
                            (unsigned long long)__double_as_longlong(v.y) & 0x7fffffffffffffffull));
         }
@@ -154,10 +161,10 @@ __global__ void oz_max_kernel(OzOp op, int R, int K, int kper, unsigned long lon
     } else {
         const int r = blockIdx.x * blockDim.x + threadIdx.x;
         if (r >= R) return;
-        const double2* x = op.X + (op.map ? (long)op.map[r] : (long)r) * op.sr;
         unsigned long long m = 0;
+#pragma unroll 4
         for (int k = k0; k < k1; ++k) {
-            const double2 v = x[(op.kmap ? (long)op.kmap[k] : (long)k) * op.sk];
+            const double2 v = op.at(r, k);
             m = max(m, max((unsigned long long)__double_as_longlong(v.x) & 0x7fffffffffffffffull,
                            (unsigned long long)__double_as_longlong(v.y) & 0x7fffffffffffffffull));
         }
@@ -208,12 +215,11 @@ __global__ void oz_fmt_kernel(OzOp op, int r0, int R, int K, int rows, int tr, i
         for (int q = 0; q < 8; ++q) d[q] = 0x0080808080808080ull;  // digits of 0
         if (r < R) {
             const double scale = __longlong_as_double((long long)(55 - oz_exp(rmax[r]) + 1023) << 52);
-            const double2* x = op.X + (op.map ? (long)op.map[r] : (long)r) * op.sr;
             const long k = (long)kb0 * OKC + 4 * ch;
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 if (k + q < K) {
-                    const double2 v = x[(op.kmap ? (long)op.kmap[k + q] : k + q) * op.sk];
+                    const double2 v = op.at(r, k + q);
                     d[2 * q] = oz_digits(v.x, scale);
                     d[2 * q + 1] = oz_digits(v.y, scale);
                 }
@@ -449,21 +455,29 @@ oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const un
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
 
-// C(m, n) = alpha sum_z part(z, n, m) + beta C(m, n), z in order
-__global__ void oz_sum_kernel(int M, int N, int splits, OzOut o) {
-    const long total = (long)M * N;
-    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-        const long n = t / M, m = t - n * M;
-        double2 s = o.part[t];
-        for (int z = 1; z < splits; ++z) s = cadd(s, o.part[(long)z * total + t]);
-        double2* c = o.C + (o.mmap ? (long)o.mmap[m] : m) * o.cm + (o.nmap ? (long)o.nmap[n] : n) * o.cn;
-        double2 v = make_double2(o.alpha * s.x, o.alpha * s.y);
-        if (o.beta != 0.0) {
-            v.x += o.beta * c->x;
-            v.y += o.beta * c->y;
-        }
-        *c = v;
+// C(m, n) = alpha sum_z part(z, n, m) + beta C(m, n): 32 outputs per block, eight groups of
+// consecutive z added in order (deterministic)
+__global__ void __launch_bounds__(256) oz_sum_kernel(int M, int N, int splits, OzOut o) {
+    __shared__ double2 sh[8][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long total = (long)M * N, t = blockIdx.x * 32l + lane;
+    const int per = (splits + 7) / 8, z1 = min(splits, (w + 1) * per);
+    double2 s = make_double2(0.0, 0.0);
+    if (t < total)
+#pragma unroll 4
+        for (int z = w * per; z < z1; ++z) s = cadd(s, o.part[(long)z * total + t]);
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w || t >= total) return;
+    for (int i = 1; i < 8; ++i) s = cadd(s, sh[i][lane]);
+    const long n = t / M, m = t - n * M;
+    double2* c = o.C + (o.mmap ? (long)o.mmap[m] : m) * o.cm + (o.nmap ? (long)o.nmap[n] : n) * o.cn;
+    double2 v = make_double2(o.alpha * s.x, o.alpha * s.y);
+    if (o.beta != 0.0) {
+        v.x += o.beta * c->x;
+        v.y += o.beta * c->y;
     }
+    *c = v;
 }
 
 inline int cdiv_(long a, long b) { return (int)((a + b - 1) / b); }
@@ -509,7 +523,8 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
         cudaFuncSetAttribute((const void*)oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, O_SMEM_MAX);
     });
     OzWork& W = c->oz;
-    const OzOp a{Am.X, Am.sr, Am.sk, Am.map, Am.kmap}, b{Bm.X, Bm.sr, Bm.sk, Bm.map, Bm.kmap};
+    const OzOp a{Am.X, Am.sr, Am.sk, Am.map, Am.kmap, Am.rp, Am.kp},
+        b{Bm.X, Bm.sr, Bm.sk, Bm.map, Bm.kmap, Bm.rp, Bm.kp};
     const int nkb = cdiv_(K, OKC), itiles = cdiv_(M, OM);
     const int jtiles = cdiv_(N, ON2_MAX / 2);
     const int tr = cdiv_(cdiv_(N, jtiles), 8) * 8, N2 = 2 * tr;  // columns of C per tile, balanced
@@ -599,6 +614,6 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
         z0 += nz;
     }
     if (ztot > 1)
-        oz_sum_kernel<<<(int)std::min<long>(2048, ((long)M * N + 255) / 256), 256, 0, c->stream>>>(M, N, ztot, o);
+        oz_sum_kernel<<<cdiv_((long)M * N, 32), 256, 0, c->stream>>>(M, N, ztot, o);
     FS_CUDA(cudaGetLastError());
 }

@@ -159,6 +159,35 @@ __global__ void herm_fill_kernel(double2* G, int n, int b1, int b2) {
     }
 }
 
+// G(i, j) = conj(G(j, i)) above the diagonal
+__global__ void herm_fill_lower_kernel(double2* G, int n) {
+    long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (t >= (long)n * n) return;
+    int i = (int)(t % n), j = (int)(t / n);
+    if (i < j) {
+        double2 v = G[(long)i * n + j];
+        G[t] = make_double2(v.x, -v.y);
+    }
+}
+
+// row pointers of a basis of up to three blocks (row r of block b: base + map(r) ld), for two
+// families of blocks (S and its images)
+template <typename T2> struct BasisRows {
+    const T2* S[3];
+    const T2* Y[3];
+    const int* map[3];
+    int off[4];
+    long ld;
+};
+template <typename T2> __global__ void basis_rows_kernel(BasisRows<T2> B, const T2** s, const T2** y) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= B.off[3]) return;
+    const int b = (r >= B.off[1]) + (r >= B.off[2]);
+    const long q = r - B.off[b], row = B.map[b] ? (long)B.map[b][q] : q;
+    s[r] = B.S[b] + row * B.ld;
+    y[r] = B.Y[b] + row * B.ld;
+}
+
 struct Solver {
     fs_ctx* c;
     double E;
@@ -193,6 +222,7 @@ struct Solver {
         s.nrm.alloc(nbmax * sizeof(double));
         s.shift.alloc(nbmax * sizeof(double));
         s.keep.alloc(2 * nbmax * sizeof(int));
+        s.rows.alloc(2 * nbmax * sizeof(void*));
     }
 
     // generalized Hermitian eigenproblem GA c = lambda GB c, n x n column-major:
@@ -432,10 +462,9 @@ struct Solver {
         T2* Y = B.Y.template as<T2>();
         T2* RH = B.RH.template as<T2>();
         T2* ZR = B.ZR.template as<T2>();
-        vec_resid<T2>(c, X, Y, m, s.hres.as<double>(), s.dots.as<double2>());
+        vec_resid<T2>(c, X, Y, m, s.hres.as<double>(), s.dots.as<double2>(), RH);
         hres_h.resize(m);
         FS_CUDA(cudaMemcpyAsync(hres_h.data(), s.hres.p, m * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        vec_rh<T2>(c, X, Y, s.dots.as<double2>(), m, RH);
         ra.resize(m);
         th.resize(m);
         if (lowest) {
@@ -559,8 +588,7 @@ struct Solver {
         }
         gemm_gram<T2>(c, m, na, npw, X, npw, nullptr, W, npw, nullptr, GB, 1, m, 1.0, 0.0);
         gemm_nn<T2, double2>(c, na, npw, m, GB, m, 1, X, npw, nullptr, W, npw, nullptr, -1.0, 1.0, W, npw);
-        vec_row_norms<T2>(c, W, nullptr, na, s.nrm.as<double>());
-        vec_scale_rows<T2>(c, W, nullptr, na, s.nrm.as<double>());
+        vec_normalize<T2>(c, W, nullptr, nullptr, na);
         HE(W, YW, na);
         bool useP = B.haveP;
         if (useP) {
@@ -568,9 +596,7 @@ struct Solver {
             gemm_gram<T2>(c, m, na, npw, X, npw, nullptr, P, npw, act, GB, 1, m, 1.0, 0.0);
             gemm_nn<T2, double2>(c, na, npw, m, GB, m, 1, X, npw, nullptr, P, npw, act, -1.0, 1.0, P, npw);
             gemm_nn<T2, double2>(c, na, npw, m, GB, m, 1, Y, npw, nullptr, YP, npw, act, -1.0, 1.0, YP, npw);
-            vec_row_norms<T2>(c, P, act, na, s.nrm.as<double>());
-            vec_scale_rows<T2>(c, P, act, na, s.nrm.as<double>());
-            vec_scale_rows<T2>(c, YP, act, na, s.nrm.as<double>());
+            vec_normalize<T2>(c, P, YP, act, na);
         }
         for (int attempt = 0; attempt < 2; ++attempt) {
             int nblk = useP ? 3 : 2;
@@ -582,8 +608,22 @@ struct Solver {
             int nb = m + na + (useP ? na : 0);
             // <s_i, A s_j> = <(H-E)s_i, (H-E)s_j>: the Y images keep the small
             // Rayleigh quotients of A accurate in the FP32 stage
-            gram_blocks<T2>(GA, nb, lowest ? S : SY, SY, maps, sizes, offs, nblk);
-            gram_blocks<T2>(GB, nb, S, S, maps, sizes, offs, nblk);
+            // (all blocks of a matrix in one product, their rows by pointers: twelve products of
+            // pairs of blocks formatted every block three times and took 0.1 ms each at 36 bands)
+            BasisRows<T2> br{{X, W, P}, {Y, YW, YP}, {nullptr, nullptr, act}, {0, m, m + na, nb}, npw};
+            const T2** rs = s.rows.as<const T2*>();
+            const T2** ry = rs + nb;
+            basis_rows_kernel<T2><<<nblk_(nb), 256, 0, c->stream>>>(br, rs, ry);
+            FS_CUDA(cudaGetLastError());
+            if (gemm_gram_rows<T2>(c, nb, (int)npw, lowest ? rs : ry, ry, GA, 1)) {
+                gemm_gram_rows<T2>(c, nb, (int)npw, rs, rs, GB, 1);
+                herm_fill_lower_kernel<<<nblk_((long)nb * nb), 256, 0, c->stream>>>(GA, nb);
+                herm_fill_lower_kernel<<<nblk_((long)nb * nb), 256, 0, c->stream>>>(GB, nb);
+                FS_CUDA(cudaGetLastError());
+            } else {
+                gram_blocks<T2>(GA, nb, lowest ? S : SY, SY, maps, sizes, offs, nblk);
+                gram_blocks<T2>(GB, nb, S, S, maps, sizes, offs, nblk);
+            }
             int info = rr_basis(nb, true, tau_for<T2>(), piv_for<T2>());
             if (info != 0) {
                 if (useP) {
@@ -602,9 +642,12 @@ struct Solver {
             dbuf* dX[2] = {&B.tX, &B.tY};
             for (int q = 0; q < 2; ++q) {
                 T2* pn = dP[q]->template as<T2>();
-                gemm_nn<T2, double2>(c, m, npw, na, V + m, nb, 1, srcW[q], npw, nullptr, pn, npw, nullptr, 1.0, 0.0,
-                                     nullptr, 0);
-                if (useP)
+                // W and P together (their rows follow one another in the pointers)
+                const bool both = gemm_nn_rows<T2>(c, m, (int)npw, nb - m, V + m, nb, (q ? ry : rs) + m, pn, npw);
+                if (!both)
+                    gemm_nn<T2, double2>(c, m, npw, na, V + m, nb, 1, srcW[q], npw, nullptr, pn, npw, nullptr, 1.0,
+                                         0.0, nullptr, 0);
+                if (!both && useP)
                     gemm_nn<T2, double2>(c, m, npw, na, V + m + na, nb, 1, srcP[q], npw, act, pn, npw, nullptr, 1.0,
                                          1.0, pn, npw);
                 gemm_nn<T2, double2>(c, m, npw, m, V, nb, 1, srcX[q], npw, nullptr, dX[q]->template as<T2>(), npw,

@@ -152,7 +152,11 @@ struct LdF2 {
     const float2* X;
     long sr, sk;
     const int *map, *kmap;
+    const float2* const* rp = nullptr;  // rows, or k, by pointers
+    const float2* const* kp = nullptr;
     __device__ __forceinline__ float2 at(int r, int k) const {
+        if (rp) return rp[r][k];
+        if (kp) return kp[k][r];
         return X[(map ? (long)map[r] : (long)r) * sr + (kmap ? (long)kmap[k] : (long)k) * sk];
     }
     __device__ __forceinline__ float mag(int r, int k) const {
@@ -358,7 +362,7 @@ struct TcOut {
 // [z kbs, min(nkb, (z + 1) kbs)).
 __global__ void __launch_bounds__(TC_THREADS, 1)
 tc_gemm_kernel(int M, int N, int m0, int N2, int itiles, int jtiles, int ntiles, int nkb, int kbs, int nst,
-               const unsigned char* __restrict__ Af, long a_stride, long a_kb0, const unsigned char* __restrict__ Bf,
+               int lower, const unsigned char* __restrict__ Af, long a_stride, long a_kb0, const unsigned char* __restrict__ Bf,
                const uint32_t* __restrict__ ma, const uint32_t* __restrict__ mb, TcOut o, int z0, int* errflag) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const uint32_t bsplit = (uint32_t)N2 * 64, sbytes = A_STAGE + 2 * bsplit;
@@ -394,6 +398,7 @@ tc_gemm_kernel(int M, int N, int m0, int N2, int itiles, int jtiles, int ntiles,
             long long g = 0;  // stages issued by this block
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
                 const int jt = tile % jtiles, it = (tile / jtiles) % itiles, kb0 = tile / (jtiles * itiles) * kbs;
+                if (lower && jt * (N2 >> 1) >= (it + 1) * TM) continue;  // wholly above the diagonal
                 const int nk = min(nkb, kb0 + kbs) - kb0;
                 const unsigned char* a = Af + ((long)it * a_stride + a_kb0 + kb0) * A_STAGE;
                 const unsigned char* b = Bf + ((long)jt * nkb + kb0) * (2l * bsplit);
@@ -419,6 +424,8 @@ tc_gemm_kernel(int M, int N, int m0, int N2, int itiles, int jtiles, int ntiles,
             long long g = 0, last = -1;
             int ch = 0;  // accumulator chains started by this block
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+                const int jt = tile % jtiles, it = (tile / jtiles) % itiles;
+                if (lower && jt * (N2 >> 1) >= (it + 1) * TM) continue;
                 const int kb0 = tile / (jtiles * itiles) * kbs, nk = min(nkb, kb0 + kbs) - kb0;
                 for (int kb = 0; kb < nk; ++kb, ++g) {
                     const int st = (int)(g % nst), buf = ch & 1;
@@ -461,6 +468,7 @@ tc_gemm_kernel(int M, int N, int m0, int N2, int itiles, int jtiles, int ntiles,
         float acc[4][32];
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
             const int jt = tile % jtiles, it = (tile / jtiles) % itiles, z = tile / (jtiles * itiles);
+            if (lower && jt * (N2 >> 1) >= (it + 1) * TM) continue;
             const int nk = min(nkb, (z + 1) * kbs) - z * kbs, nchain = (nk + CHAIN - 1) / CHAIN;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -547,27 +555,38 @@ tc_gemm_kernel(int M, int N, int m0, int N2, int itiles, int jtiles, int ntiles,
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
 
-// C(m, n) = alpha sum_z part(z, n, m) + beta C(m, n) in FP64, z in order
-__global__ void tc_sum_kernel(int M, int N, int splits, const float2* __restrict__ part, double2* C, long cm, long cn,
-                              double alpha, double beta) {
-    const long total = (long)M * N;
-    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-        double sx = 0, sy = 0;
-#pragma unroll 4
-        for (int s = 0; s < splits; ++s) {
-            const float2 v = part[(long)s * total + t];
+// C(m, n) = alpha sum_z part(z, n, m) + beta C(m, n) in FP64: 32 outputs per block, eight groups of
+// consecutive z added in order (deterministic); lower: outputs of
+// skipped tiles (tr columns wide) stay as they are
+__global__ void __launch_bounds__(256) tc_sum_kernel(int M, int N, int splits, const float2* __restrict__ part,
+                                                     double2* C, long cm, long cn, double alpha, double beta,
+                                                     int lower, int tr) {
+    __shared__ double2 sh[8][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long total = (long)M * N, t = blockIdx.x * 32l + lane;
+    const long n = t / M, m = t - n * M;
+    const bool live = t < total && !(lower && n / tr * tr >= (m / TM + 1) * TM);
+    const int per = (splits + 7) / 8, z1 = min(splits, (w + 1) * per);
+    double sx = 0, sy = 0;
+    if (live)
+#pragma unroll 8
+        for (int z = w * per; z < z1; ++z) {
+            const float2 v = part[(long)z * total + t];
             sx += v.x;
             sy += v.y;
         }
-        const long n = t / M, m = t - n * M;
-        double2* dst = C + m * cm + n * cn;
-        double2 o = make_double2(alpha * sx, alpha * sy);
-        if (beta != 0.0) {
-            o.x += beta * dst->x;
-            o.y += beta * dst->y;
-        }
-        *dst = o;
+    sh[w][lane] = make_double2(sx, sy);
+    __syncthreads();
+    if (w || !live) return;
+    double2 s = sh[0][lane];
+    for (int i = 1; i < 8; ++i) s = cadd(s, sh[i][lane]);
+    double2* dst = C + m * cm + n * cn;
+    double2 o = make_double2(alpha * s.x, alpha * s.y);
+    if (beta != 0.0) {
+        o.x += beta * dst->x;
+        o.y += beta * dst->y;
     }
+    *dst = o;
 }
 
 // The bounded wait of the pipelines, on a barrier that nothing completes: it
@@ -637,7 +656,7 @@ struct TcDst64 {
 };
 template <class OpA, class OpB>
 void tc_run(fs_ctx* c, int M, int N, int K, const OpA& a, int acont, int amaxk, const OpB& b, int bcont, int conja,
-            dbuf* keep, dbuf* keepm, const TcDst64* d64, TcOut o) {
+            dbuf* keep, dbuf* keepm, const TcDst64* d64, TcOut o, int lower = 0) {
     set_attrs();
     const int nkb = std::max(1, cdiv_(K, KC)), itiles = cdiv_(M, TM);
     const int jtiles = cdiv_(N, TN2_MAX / 2);
@@ -725,15 +744,15 @@ void tc_run(fs_ctx* c, int M, int N, int K, const OpA& a, int acont, int amaxk, 
             }
             const int ntiles = jtiles * ni * nz, grid = std::min(ntiles, g_nsm);
             tc_gemm_kernel<<<grid, TC_THREADS, (size_t)nst * sbytes + TC_CTL, c->stream>>>(
-                M, N, i0 * TM, N2, ni, jtiles, ntiles, nk, per, nst, Af, stride, akb, c->bfmt.as<unsigned char>(), ma,
+                M, N, i0 * TM, N2, ni, jtiles, ntiles, nk, per, nst, lower, Af, stride, akb, c->bfmt.as<unsigned char>(), ma,
                 mb, o, z0, ctx_errflag(c));
             FS_CUDA(cudaGetLastError());
         }
         z0 += nz;
     }
     if (d64)
-        tc_sum_kernel<<<(int)std::min<long>(2048, ((long)M * N + 127) / 128), 128, 0, c->stream>>>(
-            M, N, ztot, o.part, d64->C, d64->cm, d64->cn, d64->alpha, d64->beta);
+        tc_sum_kernel<<<cdiv_((long)M * N, 32), 256, 0, c->stream>>>(M, N, ztot, o.part, d64->C, d64->cm, d64->cn,
+                                                                     d64->alpha, d64->beta, lower, tr);
     FS_CUDA(cudaGetLastError());
 }
 
@@ -753,6 +772,22 @@ void tc_gemm_gram(fs_ctx* c, int M, int N, int K, const float2* A, long lda, con
     const LdF2 a{A, lda, 1, amap, nullptr};
     const bool table = A == c->beta32.as<float2>() && !amap && M == c->nptot && K == c->npw;
     tc_run(c, M, N, K, a, 1, K, b, 1, 1, table ? &c->beta32_gfmt : nullptr, &c->tc_gmax, &d, TcOut{});
+}
+
+void tc_gemm_gram_rows(fs_ctx* c, int n, int K, const float2* const* A, const float2* const* B, double2* C, int lower) {
+    if (n <= 0) return;
+    ProfScope ps(c, KS_GRAM, 2.0 * n * K * sizeof(float2) + (double)n * n * sizeof(double2), 8.0 * n * n * K);
+    const TcDst64 d{C, 1, n, 1.0, 0.0};
+    tc_run(c, n, n, K, LdF2{nullptr, 0, 1, nullptr, nullptr, A}, 1, K, LdF2{nullptr, 0, 1, nullptr, nullptr, B}, 1, 1,
+           nullptr, nullptr, &d, TcOut{}, lower);
+}
+
+void tc_gemm_nn_rows(fs_ctx* c, int M, int N, int K, const double2* A, long ai, const float2* const* B, float2* C,
+                     long ldc) {
+    if (M <= 0 || N <= 0) return;
+    ProfScope ps(c, KS_ROTATE, ((double)K + M) * N * sizeof(float2) + (double)M * K * sizeof(double2), 8.0 * M * N * K);
+    tc_run(c, N, M, K, LdF2{nullptr, 1, 0, nullptr, nullptr, nullptr, B}, 0, K, LdD2{A, ai, 1}, 1, 0, nullptr, nullptr,
+           nullptr, TcOut{nullptr, C, ldc, nullptr, nullptr, 0, 1.f, 0.f});
 }
 
 template <typename A2>
