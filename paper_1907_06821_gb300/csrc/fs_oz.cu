@@ -52,6 +52,7 @@ constexpr int OA_STAGE = NS * OA_SLICE;
 constexpr int O_THREADS = 320;
 constexpr int O_SMEM_MAX = 232448;
 constexpr int O_CTL = 256;
+__host__ __device__ constexpr int O_COLS(int nq) { return nq == 1 ? 256 : 512; }  // tensor-memory columns
 constexpr int O_STAGES_MAX = 8;
 constexpr int E_MIN = -900;                   // exponent of an all-zero row (components below 2^-954 read as 0)
 constexpr long long OZ_WAIT_LIMIT = 1ll << 28;
@@ -184,18 +185,71 @@ __device__ __forceinline__ uint32_t oz_pair(unsigned long long p, unsigned long 
     return __byte_perm(__float_as_uint(fp), __float_as_uint(fq), 0x7632);
 }
 
-// One thread writes the 16-byte chunk (4 complex k) of one row in every slice.
-//   BSIDE = false: A image, rows r0 + local row, tiles of 128 rows
+// The 16-byte chunk ch (4 complex k) of local row lr (operand row r) in every slice.
+//   BSIDE = false: A image, tiles of 128 rows
 //   BSIDE = true : B image, tiles of tr = N2 / 2 operand rows, two image rows each;
 //                  conja / conjb: conjugated A and B of the product
-// Stages [kb0, kb0 + nkb) of the operand become local stages 0 .. nkb.
+template <bool BSIDE>
+__device__ __forceinline__ void oz_put(const OzOp& op, int lr, int r, int R, long ch, int K, int tr, int kb0, int nkb,
+                                       int conja, int conjb, double scale, unsigned char* __restrict__ out) {
+    const uint32_t slice = BSIDE ? (uint32_t)tr * 64 : (uint32_t)OA_SLICE;
+    unsigned long long d[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) d[q] = 0x0080808080808080ull;  // digits of 0
+    if (r < R) {
+        const long k = (long)kb0 * OKC + 4 * ch;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (k + q < K) {
+                const double2 v = op.at(r, k + q);
+                d[2 * q] = oz_digits(v.x, scale);
+                d[2 * q + 1] = oz_digits(v.y, scale);
+            }
+    }
+    const long kb = ch >> 1;
+    const int half = (int)(ch & 1);
+    if (!BSIDE) {
+        unsigned char* st = out + ((long)(lr / OM) * nkb + kb) * OA_STAGE + oz_chunk(lr % OM, half);
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+            *reinterpret_cast<uint4*>(st + s * OA_SLICE) =
+                make_uint4(oz_pair(d[0], d[1], NS - 1 - s), oz_pair(d[2], d[3], NS - 1 - s),
+                           oz_pair(d[4], d[5], NS - 1 - s), oz_pair(d[6], d[7], NS - 1 - s));
+    } else {
+        // b' = conjb ? conj(b) : b; rows (b'r, -b'i), (b'i, b'r), or with conja (b'r, b'i), (b'i, -b'r)
+        const uint32_t s0 = (conja != 0) == (conjb != 0) ? 0x80000000u : 0u;  // sign of the im half, first row
+        const uint32_t s1l = conjb ? 0x00008000u : 0u;                        // sign of im, second row
+        const uint32_t s1h = conja ? 0x80000000u : 0u;                        // sign of re, second row
+        const int tile = lr / tr, j = lr - tile * tr;
+        unsigned char* st = out + ((long)tile * nkb + kb) * ((long)NS * slice);
+        const uint32_t o0 = oz_chunk(2 * j, half);
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            uint32_t a[4], b[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t p = oz_pair(d[2 * q], d[2 * q + 1], NS - 1 - s);  // (re, im)
+                a[q] = p ^ s0;
+                b[q] = __byte_perm(p, p, 0x1032) ^ (s1l | s1h);                   // (im, re)
+            }
+            unsigned char* sl = st + (long)s * slice;
+            *reinterpret_cast<uint4*>(sl + o0) = make_uint4(a[0], a[1], a[2], a[3]);
+            *reinterpret_cast<uint4*>(sl + o0 + 16) = make_uint4(b[0], b[1], b[2], b[3]);
+        }
+    }
+}
+
+__device__ __forceinline__ double oz_scale(unsigned long long bits) {
+    return __longlong_as_double((long long)(55 - oz_exp(bits) + 1023) << 52);
+}
+
+// Rows r0 .., stages [kb0, kb0 + nkb) of the operand as local stages 0 .. nkb, by known maxima
 template <bool BSIDE>
 __global__ void oz_fmt_kernel(OzOp op, int r0, int R, int K, int rows, int tr, int kb0, int nkb, int conja, int conjb,
                               const unsigned long long* __restrict__ rmax, unsigned char* __restrict__ out) {
     const bool kcont = op.sk == 1;
     const long nch = 2l * nkb;  // chunks of 4 complex k per row
     const long total = kcont ? (long)(rows / 8) * ((nch + 3) / 4) * 32 : (long)rows * nch;
-    const uint32_t slice = BSIDE ? (uint32_t)tr * 64 : (uint32_t)OA_SLICE;
     for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
         int lr;   // local row
         long ch;  // local chunk
@@ -210,51 +264,54 @@ __global__ void oz_fmt_kernel(OzOp op, int r0, int R, int K, int rows, int tr, i
             ch = t / rows;
         }
         const int r = r0 + lr;
-        unsigned long long d[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) d[q] = 0x0080808080808080ull;  // digits of 0
-        if (r < R) {
-            const double scale = __longlong_as_double((long long)(55 - oz_exp(rmax[r]) + 1023) << 52);
-            const long k = (long)kb0 * OKC + 4 * ch;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (k + q < K) {
-                    const double2 v = op.at(r, k + q);
-                    d[2 * q] = oz_digits(v.x, scale);
-                    d[2 * q + 1] = oz_digits(v.y, scale);
-                }
+        oz_put<BSIDE>(op, lr, r, R, ch, K, tr, kb0, nkb, conja, conjb, r < R ? oz_scale(rmax[r]) : 0.0, out);
+    }
+}
+
+// Maxima and images in one launch, all K.  Rows along k (short ones): 8 rows per block, a warp
+// finds a row's maximum.  Rows contiguous in memory: 32 rows per block, a warp takes every
+// eighth k, then every eighth chunk.  (Three launches an operand made a small product 60 us.)
+template <bool BSIDE>
+__global__ void __launch_bounds__(256) oz_maxfmt_kernel(OzOp op, int r0, int R, int K, int rows, int tr, int nkb,
+                                                        int conja, int conjb, unsigned long long* __restrict__ rmax,
+                                                        unsigned char* __restrict__ out) {
+    __shared__ unsigned long long part[8][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto mag = [&](int r, int k) {
+        const double2 v = op.at(r, k);
+        return max((unsigned long long)__double_as_longlong(v.x) & 0x7fffffffffffffffull,
+                   (unsigned long long)__double_as_longlong(v.y) & 0x7fffffffffffffffull);
+    };
+    unsigned long long m = 0;
+    if (op.sk == 1) {
+        const int lr0 = blockIdx.x * 8, r = r0 + lr0 + w;
+        if (r < R)
+#pragma unroll 4
+            for (int k = lane; k < K; k += 32) m = max(m, mag(r, k));
+        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0) {
+            part[0][w] = m;
+            if (r < R) rmax[r] = m;
         }
-        const long kb = ch >> 1;
-        const int half = (int)(ch & 1);
-        if (!BSIDE) {
-            unsigned char* st = out + ((long)(lr / OM) * nkb + kb) * OA_STAGE + oz_chunk(lr % OM, half);
-#pragma unroll
-            for (int s = 0; s < NS; ++s)
-                *reinterpret_cast<uint4*>(st + s * OA_SLICE) =
-                    make_uint4(oz_pair(d[0], d[1], NS - 1 - s), oz_pair(d[2], d[3], NS - 1 - s),
-                               oz_pair(d[4], d[5], NS - 1 - s), oz_pair(d[6], d[7], NS - 1 - s));
-        } else {
-            // b' = conjb ? conj(b) : b; rows (b'r, -b'i), (b'i, b'r), or with conja (b'r, b'i), (b'i, -b'r)
-            const uint32_t s0 = (conja != 0) == (conjb != 0) ? 0x80000000u : 0u;  // sign of the im half, first row
-            const uint32_t s1l = conjb ? 0x00008000u : 0u;                        // sign of im, second row
-            const uint32_t s1h = conja ? 0x80000000u : 0u;                        // sign of re, second row
-            const int tile = lr / tr, j = lr - tile * tr;
-            unsigned char* st = out + ((long)tile * nkb + kb) * ((long)NS * slice);
-            const uint32_t o0 = oz_chunk(2 * j, half);
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                uint32_t a[4], b[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint32_t p = oz_pair(d[2 * q], d[2 * q + 1], NS - 1 - s);  // (re, im)
-                    a[q] = p ^ s0;
-                    b[q] = __byte_perm(p, p, 0x1032) ^ (s1l | s1h);                   // (im, re)
-                }
-                unsigned char* sl = st + (long)s * slice;
-                *reinterpret_cast<uint4*>(sl + o0) = make_uint4(a[0], a[1], a[2], a[3]);
-                *reinterpret_cast<uint4*>(sl + o0 + 16) = make_uint4(b[0], b[1], b[2], b[3]);
-            }
+        __syncthreads();
+        for (int t = threadIdx.x; t < 16 * nkb; t += 256) {
+            const int lr = lr0 + (t & 7);
+            oz_put<BSIDE>(op, lr, r0 + lr, R, t >> 3, K, tr, 0, nkb, conja, conjb, oz_scale(part[0][t & 7]), out);
         }
+    } else {
+        const int lr = blockIdx.x * 32 + lane, r = r0 + lr;
+        if (r < R)
+#pragma unroll 4
+            for (int k = w; k < K; k += 8) m = max(m, mag(r, k));
+        part[w][lane] = m;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) m = max(m, part[i][lane]);
+        if (w == 0 && r < R) rmax[r] = m;
+        const double s = oz_scale(m);
+        if (lr < rows)
+            for (int ch = w; ch < 2 * nkb; ch += 8)
+                oz_put<BSIDE>(op, lr, r, R, ch, K, tr, 0, nkb, conja, conjb, s, out);
     }
 }
 
@@ -271,7 +328,11 @@ struct OzOut {
 // each (34 digit pairs i + j <= 7 into accumulator i + j), warps 2-9 drain the eight
 // accumulators of a chain (thread: row 32 (warp & 3) + lane, half of the columns).
 // Two accumulator sets when 16 N2 <= 512 columns of tensor memory, else one.
-__global__ void __launch_bounds__(O_THREADS, 1)
+// NQ: groups of 8 accumulator columns per drain thread (N2 <= 16 NQ).  With one group (at most
+// eight columns of C) two blocks fit on an SM (registers, tensor memory, half the ring each), so
+// that one's start and epilogue run under the other's copies.
+template <int NQ>
+__global__ void __launch_bounds__(O_THREADS, NQ == 1 ? 2 : 1)
 oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const unsigned char* __restrict__ Af,
                long a_stride, long a_kb0, const unsigned char* __restrict__ Bf, const unsigned long long* __restrict__ ma,
                const unsigned long long* __restrict__ mb, OzOut o, int z0, int* errflag) {
@@ -295,7 +356,7 @@ oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const un
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(oz_smem(tslot)), "r"(512));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(oz_smem(tslot)), "r"(O_COLS(NQ)));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -304,7 +365,7 @@ oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const un
     const uint32_t tmem = *tslot;
     const int jt = blockIdx.x, it = blockIdx.y, z = blockIdx.z;
     const int kb0 = z * kbs, nk = min(nkb, kb0 + kbs) - kb0;
-    const int nbuf = 2 * ND * N2 <= 512 ? 2 : 1;
+    const int nbuf = 2 * ND * N2 <= O_COLS(NQ) ? 2 : 1;
     const int nchain = (nk + OCHAIN - 1) / OCHAIN;
     const unsigned char* a = Af + ((long)it * a_stride + a_kb0 + kb0) * OA_STAGE;
     const unsigned char* b = Bf + ((long)jt * nkb + kb0) * (long)bstage;
@@ -377,9 +438,9 @@ oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const un
     } else {
         const int q = warp & 3, h = (warp - 2) >> 2;
         const int nq = N2 >> 4;  // groups of 8 accumulator columns of this half
-        long long hi[4][8], lo[4][8];
+        long long hi[NQ][8], lo[NQ][8];
 #pragma unroll
-        for (int g = 0; g < 4; ++g)
+        for (int g = 0; g < NQ; ++g)
 #pragma unroll
             for (int e = 0; e < 8; ++e) hi[g][e] = lo[g][e] = 0;
         for (int ch = 0; ch < nchain; ++ch) {
@@ -392,7 +453,7 @@ oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const un
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * ND * N2 + h * (N2 >> 1));
 #pragma unroll
-            for (int g = 0; g < 4; ++g)
+            for (int g = 0; g < NQ; ++g)
                 if (g < nq) {  // warp-uniform
                     uint32_t r[ND][8];
 #pragma unroll
@@ -417,7 +478,7 @@ oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const un
             const unsigned long long am = ma[m];
             const int ea = oz_exp(am);
 #pragma unroll
-            for (int g = 0; g < 4; ++g)
+            for (int g = 0; g < NQ; ++g)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int jj = h * (N2 >> 2) + 4 * g + e, n = jt * (N2 >> 1) + jj;
@@ -452,7 +513,7 @@ oz_gemm_kernel(int M, int N, int m0, int N2, int nkb, int kbs, int nst, const un
     if (!ok) *(volatile int*)errflag = 1;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(O_COLS(NQ)));
 }
 
 // C(m, n) = alpha sum_z part(z, n, m) + beta C(m, n): 32 outputs per block, eight groups of
@@ -492,6 +553,13 @@ void row_max(fs_ctx* c, const OzOp& op, int R, int K, unsigned long long* out) {
 }
 
 template <bool BSIDE>
+void maxfmt(fs_ctx* c, const OzOp& op, int r0, int R, int K, int rows, int tr, int nkb, int conja, int conjb,
+            unsigned long long* rmax, unsigned char* out) {
+    oz_maxfmt_kernel<BSIDE><<<op.sk == 1 ? rows / 8 : cdiv_(rows, 32), 256, 0, c->stream>>>(
+        op, r0, R, K, rows, tr, nkb, conja, conjb, rmax, out);
+}
+
+template <bool BSIDE>
 void fmt(fs_ctx* c, const OzOp& op, int r0, int R, int K, int rows, int tr, int kb0, int nkb, int conja, int conjb,
          const unsigned long long* rmax, unsigned char* out) {
     // whole warps: 8 rows x 4 chunks
@@ -520,7 +588,9 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
     table = std::max(table, 0);
     const int conja = Am.conj, conjb = Bm.conj;
     std::call_once(g_oz_attr, [] {
-        cudaFuncSetAttribute((const void*)oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, O_SMEM_MAX);
+        for (const void* k : {(const void*)oz_gemm_kernel<1>, (const void*)oz_gemm_kernel<2>,
+                              (const void*)oz_gemm_kernel<4>})
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, O_SMEM_MAX);
     });
     OzWork& W = c->oz;
     const OzOp a{Am.X, Am.sr, Am.sk, Am.map, Am.kmap, Am.rp, Am.kp},
@@ -537,21 +607,14 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
     W.mb.ensure((size_t)N * sizeof(unsigned long long));
     unsigned long long* ma = W.ma.as<unsigned long long>();
     unsigned long long* mb = W.mb.as<unsigned long long>();
-    if (keep) {
-        if (!keep->p) {
-            keepm->ensure((size_t)M * sizeof(unsigned long long));
-            keep->alloc(abytes);
-            row_max(c, a, M, K, keepm->as<unsigned long long>());
-            fmt<false>(c, a, 0, M, K, itiles * OM, 0, 0, nkb, 0, 0, keepm->as<unsigned long long>(),
-                       keep->as<unsigned char>());
-        }
-        ma = keepm->as<unsigned long long>();
-    } else {
-        row_max(c, a, M, K, ma);
-    }
-    row_max(c, b, N, K, mb);
-    // stages per chunk and row tiles per chunk of the per-call images (at most OZ_CHUNK_BYTES each)
     const size_t OZ_CHUNK_BYTES = 1ull << 30;
+    // an operand is scaled and formatted in one launch (all of K at once) while that leaves a block
+    // at most 16,384 elements (8 rows along k, 32 rows contiguous in memory) or there are blocks for
+    // every SM; else maxima first, and by chunks of k.  (64 rows of 5,514 in eight blocks took 100 us
+    // longer than three launches.)
+    const bool onea = a.sk == 1 ? K <= 2048 || (K <= 8192 && M >= 8 * 152) : K <= 512 || M >= 32 * 152;
+    const bool oneb = b.sk == 1 ? K <= 2048 || (K <= 8192 && N >= 8 * 152) : K <= 512 || N >= 32 * 152;
+    // stages per chunk and row tiles per chunk of the per-call images (at most OZ_CHUNK_BYTES each)
     int kch = nkb, ich = itiles;
     if (!keep) {
         // long rows (Gram form): chunks of k; many rows (apply form): chunks of rows
@@ -563,11 +626,29 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
     kch = (int)std::max<size_t>(64, std::min<size_t>(kch, OZ_CHUNK_BYTES / (bstage * jtiles)));
     kch = std::min(nkb, cdiv_(kch, OCHAIN) * OCHAIN);
     if (kch < nkb) ich = itiles;
+    const bool whole = kch == nkb;
+    if (keep) {
+        if (!keep->p) {
+            keepm->ensure((size_t)M * sizeof(unsigned long long));
+            keep->alloc(abytes);
+            unsigned long long* mx = keepm->as<unsigned long long>();
+            if (onea) {
+                maxfmt<false>(c, a, 0, M, K, itiles * OM, 0, nkb, 0, 0, mx, keep->as<unsigned char>());
+            } else {
+                row_max(c, a, M, K, mx);
+                fmt<false>(c, a, 0, M, K, itiles * OM, 0, 0, nkb, 0, 0, mx, keep->as<unsigned char>());
+            }
+        }
+        ma = keepm->as<unsigned long long>();
+    } else if (!(onea && whole)) {
+        row_max(c, a, M, K, ma);
+    }
+    if (!(oneb && whole)) row_max(c, b, N, K, mb);
     // split of a chunk's stages over the grid's z: fill the SMs, whole chains per split
     auto splits_of = [&](int nk) {
         const int tiles = jtiles * std::min(ich, itiles);
-        const int want = std::max(1, 152 / tiles);
-        return std::max(1, std::min({want, nk / (4 * OCHAIN), 4096}));
+        const int want = std::max(1, (N2 <= 16 ? 2 : 1) * 152 / tiles);
+        return std::max(1, std::min({want, nk / (2 * OCHAIN), 4096}));
     };
     std::vector<int> zs;
     int ztot = 0;
@@ -582,12 +663,16 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
         o.part = W.part.as<double2>();
     }
     const size_t sbytes = OA_STAGE + bstage;
-    const int nst = (int)std::min<size_t>(O_STAGES_MAX, (O_SMEM_MAX - O_CTL) / sbytes);
+    const auto kernel = N2 <= 16 ? oz_gemm_kernel<1> : N2 <= 32 ? oz_gemm_kernel<2> : oz_gemm_kernel<4>;
+    const int nst = (int)std::min<size_t>(O_STAGES_MAX, ((N2 <= 16 ? 112 * 1024 : O_SMEM_MAX) - O_CTL) / sbytes);
     int z0 = 0, q = 0;
     for (int k0 = 0; k0 < nkb; k0 += kch, ++q) {
         const int nk = std::min(kch, nkb - k0), per = zs[q], nz = cdiv_(nk, per);
         W.bimg.ensure((size_t)jtiles * nk * bstage);
-        fmt<true>(c, b, 0, N, K, jtiles * tr, tr, k0, nk, conja, conjb, mb, W.bimg.as<unsigned char>());
+        if (oneb && whole)
+            maxfmt<true>(c, b, 0, N, K, jtiles * tr, tr, nkb, conja, conjb, mb, W.bimg.as<unsigned char>());
+        else
+            fmt<true>(c, b, 0, N, K, jtiles * tr, tr, k0, nk, conja, conjb, mb, W.bimg.as<unsigned char>());
         for (int i0 = 0; i0 < itiles; i0 += ich) {
             const int ni = std::min(ich, itiles - i0);
             const unsigned char* Af;
@@ -598,14 +683,17 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
                 akb = k0;
             } else {
                 W.aimg.ensure((size_t)ni * nk * OA_STAGE);
-                fmt<false>(c, a, i0 * OM, M, K, ni * OM, 0, k0, nk, 0, 0, ma, W.aimg.as<unsigned char>());
+                if (onea && whole)
+                    maxfmt<false>(c, a, i0 * OM, M, K, ni * OM, 0, nkb, 0, 0, ma, W.aimg.as<unsigned char>());
+                else
+                    fmt<false>(c, a, i0 * OM, M, K, ni * OM, 0, k0, nk, 0, 0, ma, W.aimg.as<unsigned char>());
                 Af = W.aimg.as<unsigned char>();
                 stride = nk;
                 akb = 0;
             }
             for (int y0 = 0; y0 < ni; y0 += 65535) {
                 const int ny = std::min(65535, ni - y0);
-                oz_gemm_kernel<<<dim3(jtiles, ny, nz), O_THREADS, (size_t)nst * sbytes + O_CTL, c->stream>>>(
+                kernel<<<dim3(jtiles, ny, nz), O_THREADS, (size_t)nst * sbytes + O_CTL, c->stream>>>(
                     M, N, (i0 + y0) * OM, N2, nk, per, nst, Af + (size_t)y0 * stride * OA_STAGE, stride, akb,
                     W.bimg.as<unsigned char>(), ma, mb, o, z0, ctx_errflag(c));
             }
