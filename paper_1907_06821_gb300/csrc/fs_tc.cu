@@ -147,7 +147,17 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
 
 // ---------------------------------------------------------------- operands
 // element (r, k) of a GEMM operand: strided with optional row and k maps, or formed from the
-// generated projectors (rows = projectors or rows = plane waves)
+// generated projectors (rows = projectors or rows = plane waves).  load4: elements k .. k + 3 of
+// row r, zeros beyond R and K; called by whole warps whose lanes 4 i .. 4 i + 3 hold consecutive
+// rows (a multiple of 4 first) of one chunk when rows are walked along k
+template <class Op>
+__device__ __forceinline__ void load4_each(const Op& op, int r, int R, int k, int K, float2 (&v)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        v[q] = make_float2(0.f, 0.f);
+        if (r < R && k + q < K) v[q] = op.at(r, k + q);
+    }
+}
 struct LdF2 {
     const float2* X;
     long sr, sk;
@@ -162,6 +172,9 @@ struct LdF2 {
     __device__ __forceinline__ float mag(int r, int k) const {
         const float2 v = at(r, k);
         return fmaxf_nan(fabsf(v.x), fabsf(v.y));
+    }
+    __device__ __forceinline__ void load4(int r, int R, int k, int K, float2 (&v)[4]) const {
+        load4_each(*this, r, R, k, K, v);
     }
     __device__ static __forceinline__ float fmaxf_nan(float a, float b) {  // NaN wins
         return __uint_as_float(max(__float_as_uint(a), __float_as_uint(b)));
@@ -178,9 +191,41 @@ struct LdD2 {
         const float2 v = at(r, k);
         return LdF2::fmaxf_nan(fabsf(v.x), fabsf(v.y));
     }
+    __device__ __forceinline__ void load4(int r, int R, int k, int K, float2 (&v)[4]) const {
+        load4_each(*this, r, R, k, K, v);
+    }
 };
+// phase e^{-i q_g.R_a} of atom a at plane wave g
+__device__ __forceinline__ float2 gen_phase(const BetaGen& B, int a, int g) {
+    const int code = B.gidx[g];
+    const float2* ph = B.ph32 + (long)a * 3 * B.span;
+    return cmul(cmul(ph[code & 1023], ph[B.span + ((code >> 10) & 1023)]), ph[2 * B.span + ((code >> 20) & 1023)]);
+}
+// radial factor times phase (times -i for a p type)
+__device__ __forceinline__ float2 gen_value(float r, float2 e, bool p) {
+    return p ? make_float2(r * e.y, -r * e.x) : make_float2(r * e.x, r * e.y);
+}
 struct LdGenP {  // rows: projectors
     BetaGen B;
+    // the projectors of an atom share its phases: with a multiple of 4 per atom, four lanes on
+    // four projectors of one atom form one phase each and exchange them (the phases were three
+    // quarters of the arithmetic: H application of 96 bands of the long wire 136 -> 91 ms)
+    __device__ __forceinline__ void load4(int r, int R, int k, int K, float2 (&v)[4]) const {
+        if (B.nproj & 3) {
+            load4_each(*this, r, R, k, K, v);
+            return;
+        }
+        const int lane = threadIdx.x & 31, rr = min(r, R - 1), a = rr / B.nproj, c = rr - a * B.nproj;
+        const float2 mine = gen_phase(B, a, min(k + (lane & 3), K - 1));
+        const bool p = B.pl[c] != 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int src = (lane & ~3) | q;
+            const float2 e = make_float2(__shfl_sync(0xffffffffu, mine.x, src), __shfl_sync(0xffffffffu, mine.y, src));
+            v[q] = make_float2(0.f, 0.f);
+            if (r < R && k + q < K) v[q] = gen_value(B.rad32[(long)c * B.npw + k + q], e, p);
+        }
+    }
     __device__ __forceinline__ float2 at(int r, int k) const { return beta_value32(B, r, k); }
     // (the phase has modulus one up to rounding)
     __device__ __forceinline__ float mag(int r, int k) const {
@@ -189,6 +234,20 @@ struct LdGenP {  // rows: projectors
 };
 struct LdGenG {  // rows: plane waves
     BetaGen B;
+    // four projectors of one atom: one phase
+    __device__ __forceinline__ void load4(int r, int R, int k, int K, float2 (&v)[4]) const {
+        if (B.nproj & 3) {
+            load4_each(*this, r, R, k, K, v);
+            return;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = make_float2(0.f, 0.f);
+        if (r >= R || k >= K) return;
+        const int a = k / B.nproj, c = k - a * B.nproj;
+        const float2 e = gen_phase(B, a, r);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = gen_value(B.rad32[(long)(c + q) * B.npw + r], e, B.pl[c + q] != 0);
+    }
     __device__ __forceinline__ float2 at(int r, int k) const { return beta_value32(B, k, r); }
     __device__ __forceinline__ float mag(int r, int k) const {
         return 1.0001f * fabsf(B.rad32[(long)(k % B.nproj) * B.npw + r]);
@@ -239,11 +298,7 @@ __device__ __forceinline__ void put_chunk(const Op& op, int lr, int r, int R, in
     const uint32_t split = BSIDE ? (uint32_t)tr * 128 : (uint32_t)A_SPLIT;
     const int k = kb0 * KC + 4 * ch;
     float2 v[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        v[q] = make_float2(0.f, 0.f);
-        if (r < R && k + q < K) v[q] = op.at(r, k + q);
-    }
+    op.load4(r, R, k, K, v);
     uint32_t h[4], l[4];  // (re, im) pairs of the hi and lo parts
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -637,6 +692,18 @@ template <class Op> void tc_row_max(fs_ctx* c, const Op& op, int kcont, int R, i
     tc_max_kernel<Op><<<dim3(bx, by), 256, 0, c->stream>>>(op, R, K, cdiv_(K, by), kcont, out);
 }
 
+// maxima of the first `have` rows repeated over the others
+__global__ void tc_repeat_kernel(uint32_t* m, int have, int R) {
+    const int r = have + blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < R) m[r] = m[r % have];
+}
+// projectors of one type have the same radial factor: nproj rows stand for all
+void tc_row_max(fs_ctx* c, const LdGenP& op, int kcont, int R, int K, uint32_t* out) {
+    const int have = std::min(R, op.B.nproj);
+    tc_row_max<LdGenP>(c, op, kcont, have, K, out);
+    if (R > have) tc_repeat_kernel<<<cdiv_(R - have, 256), 256, 0, c->stream>>>(out, have, R);
+}
+
 template <bool BSIDE, class Op>
 void tc_fmt(fs_ctx* c, const Op& op, int kcont, int r0, int R, int K, int rows, int tr, int kb0, int nkb, int conja,
             const uint32_t* rmax, unsigned char* out) {
@@ -700,11 +767,26 @@ void tc_run(fs_ctx* c, int M, int N, int K, const OpA& a, int acont, int amaxk, 
                                                                                    jtiles * bstage)));
     else if (!d64 && !keep)
         ich = (int)std::max<size_t>(1, std::min<size_t>(itiles, FS_FMT_CHUNK_BYTES / ((size_t)nkb * A_STAGE)));
-    // split of a chunk over K: about two tiles per SM, at least two chains each
+    // split of a chunk over K (at least two chains each): the fewest splits with which the tiles
+    // come to whole rounds over the SMs but for 7 %, else those with the least idle time (48
+    // tiles of the wire's projections: 3 splits = 144 tiles instead of 7 = 336, which left the
+    // third round of blocks a fifth full)
+    const int tiles = lower ? std::max(1, (itiles * jtiles + std::max(itiles, jtiles)) / 2) : itiles * jtiles;
     auto per_split = [&](int nk) {
-        const int want = std::max(1, cdiv_(2 * g_nsm, itiles * jtiles));
-        const int splits = d64 ? std::max(1, std::min(want, nk / (2 * CHAIN))) : 1;
-        return cdiv_(nk, splits);
+        int best = 1;
+        if (d64) {
+            double eff_best = 0;
+            const int most = std::max(1, std::min(nk / (2 * CHAIN), cdiv_(4 * g_nsm, tiles)));
+            for (int sp = 1; sp <= most; ++sp) {
+                const double eff = (double)tiles * sp / ((double)cdiv_((long)tiles * sp, g_nsm) * g_nsm);
+                if (eff > eff_best + 1e-9) {
+                    eff_best = eff;
+                    best = sp;
+                }
+                if (eff >= 0.93) break;
+            }
+        }
+        return cdiv_(nk, best);
     };
     int ztot = 0;
     if (d64) {
