@@ -33,6 +33,30 @@ template <typename T2, typename R> __host__ __device__ __forceinline__ T2 cscale
     return mk(a.x * s, a.y * s);
 }
 
+// float2 sums on the packed FP32 instructions (two additions an instruction)
+__device__ __forceinline__ unsigned long long pack2(float2 a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long r) {
+    float2 a;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+    return a;
+}
+__device__ __forceinline__ float2 padd(float2 a, float2 b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 psub(float2 a, float2 b) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ double2 padd(double2 a, double2 b) { return cadd(a, b); }
+__device__ __forceinline__ double2 psub(double2 a, double2 b) { return csub(a, b); }
+
 template <typename T2> struct real_of;
 template <> struct real_of<double2> { using t = double; };
 template <> struct real_of<float2> { using t = float; };
