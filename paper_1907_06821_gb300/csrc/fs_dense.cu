@@ -374,9 +374,12 @@ hetrd_kernel(int n, double2* A, double2* V, double2* tau, double* d, double* e, 
             const double s2 = fma(al.x, al.x, fma(al.y, al.y, xn2));
             double ib, id, dx;
             if (s2 > 0x1p-900 && s2 < 0x1p+900) {
-                const double rs = newton_rsqrt(s2);
-                ib = -copysign(rs, al.x);
-                beta = s2 * ib;  // -sign(Re alpha) sqrt(s2)
+                // square root and its reciprocal corrected to their last bit (a reflector is unitary
+                // to the accuracy of these two)
+                const double rs = newton_rsqrt(s2), q0 = s2 * rs;
+                const double nrm = fma(0.5 * rs, fma(-q0, q0, s2), q0);
+                beta = -copysign(nrm, al.x);
+                ib = -copysign(fma(rs, fma(-nrm, rs, 1.0), rs), al.x);
                 dx = al.x - beta;
                 id = newton_rcp(fma(dx, dx, al.y * al.y));
             } else {
