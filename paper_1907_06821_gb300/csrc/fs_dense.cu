@@ -272,11 +272,11 @@ __global__ void hermitize_kernel(double2* A, int n) {
 // own flags: Y and C have a row per step, filled with a NaN pattern beforehand, and the
 // readers poll until every entry has changed, so a step costs one store and one load
 // through L2 instead of a grid barrier, a segment sum and three reads of A.
-// Bound: FP64 rate (12 operations per element of A22 and step, 20 per row and block) and
+// Bound: FP64 rate (14 operations per element of A22 and step, 20 per row and block) and
 // about 6 us a step of dependent FP64 operations and L2 round trips.  Four warps, one per
 // scheduler: what every warp computes for itself (the reflector's scalars, the sums) then
 // costs its own pipe only; eight took 45 % longer at n = 108.  Measured: n = 816: 20.0 ->
-// 13.5 ms, n = 204: 2.3 -> 1.5 ms.
+// 14.4 ms, n = 204: 2.3 -> 1.6 ms.
 constexpr unsigned long long EMPTY = 0xffffffffffffffffull;     // a NaN that no arithmetic returns
 
 __device__ __forceinline__ void publish(double* p, double v) {
@@ -422,8 +422,9 @@ hetrd_kernel(int n, double2* A, double2* V, double2* tau, double* d, double* e, 
                 if (r > i && r < n) {
                     double2 a = col[r];
                     if (i > 0) {  // a -= v conj(wj) + w conj(vj)
-                        a.x = fma(-v[q].x, wj.x, fma(-v[q].y, wj.y, fma(-w[q].x, vj.x, fma(-w[q].y, vj.y, a.x))));
-                        a.y = fma(v[q].x, wj.y, fma(-v[q].y, wj.x, fma(w[q].x, vj.y, fma(-w[q].y, vj.x, a.y))));
+                        // (the term by itself first: one rounding at the size of a, not four)
+                        a.x -= fma(v[q].x, wj.x, fma(v[q].y, wj.y, fma(w[q].x, vj.x, w[q].y * vj.y)));
+                        a.y -= fma(v[q].y, wj.x, fma(-v[q].x, wj.y, fma(w[q].y, vj.x, -w[q].x * vj.y)));
                         col[r] = a;
                     }
                     if (j == i + 1) {
