@@ -35,16 +35,11 @@ import numpy as np  # noqa: E402
 
 # DRAM traffic over algorithmic bytes for one launch, from one ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum) of the medium profiling case (64 bands, 512 projectors, 41,657 plane waves;
-# profiles/tcq_kernels_medium_64bands.md).  The formatted operand images are the reason it exceeds 1:
-# the projector table is read as TF32 hi and lo images (2x), expanded to 2x2 real blocks for the add (4x).
+# profiles/tc_gemm_kernel_medium_64bands.md): the projector table is read as FP16 hi and lo images of
+# its FP32 size, the add reads and writes the bands besides.
 NCU_TRAFFIC_RATIO = {
-    "nonlocal_project": (426.996736e6 + 14.766592e6) / ((512 + 64) * 41657 * 8 + 512 * 64 * 16),
-    "nonlocal_add": (706.371584e6 + 18.200576e6) / ((512 + 2 * 64) * 41657 * 8 + 64 * 512 * 16),
-    # the same ratio for a Gram matrix of two 136-band blocks and for the in-place projection
-    # W -= X (X^H W) of 136 bands, from the bounded medium solve (profiles/tcq_gram_kernel_medium_solve.md,
-    # profiles/tcq_nn_kernel_medium_solve.md): formatted images read once, tile re-reads from L2
-    "gram": (362.928896e6 + 10.022144e6) / ((136 + 136) * 41657 * 8 + 136 * 136 * 16),
-    "rotate": (227.311360e6 + 16.754176e6) / ((136 + 2 * 136) * 41657 * 8 + 136 * 136 * 16),
+    "nonlocal_project": (213.795584e6 + 3.955712e6) / ((512 + 64) * 41657 * 8 + 512 * 64 * 16),
+    "nonlocal_add": (194.109696e6 + 2.042624e6) / ((512 + 2 * 64) * 41657 * 8 + 64 * 512 * 16),
 }
 METRIC = "states converged/s to 1e-6 residual (mixed+learned vs plain FP64); Hψ HBM GB/s"
 TOL = 1e-6
@@ -362,9 +357,9 @@ def make_line(args, w, ctx, results, stats, nconv, tmax, t_e2e, e2e_states, cloc
     traffic = NCU_TRAFFIC_RATIO[top] * avg_bytes if top in NCU_TRAFFIC_RATIO else None
     if top in ("gram", "rotate", "nonlocal_project", "nonlocal_add"):
         if fp32:
-            # tcgen05 kind::tf32 with a 3-term split: TF32 peak = measured BF16 peak x nominal TF32/BF16 ratio
-            cpeak, cbound = bf16 * (1.1 / 2.25), "tensor"
-            csrc = f"{src} bf16_tflops x 1.1/2.25 (TF32); the TF32 x3 split runs 3 MMAs per product"
+            # tcgen05 kind::f16 with a two-part FP16 split
+            cpeak, cbound = bf16, "tensor"
+            csrc = f"{src} bf16_tflops; the FP16 split runs 3 MMAs per product"
         else:
             cpeak, cbound = 152 * 128 * 2 * 2.07e9 / 1e12 / 64, "alu"
             csrc = "FP64 CUDA-core peak 152 SMs x 64 FMA x 2 x 2.07 GHz / 64 (GB300 FP64 rate)"

@@ -5,11 +5,11 @@
 //                for B, T (transpose);
 //                16 x 16 tiles staged in shared memory (FP64 FMA), or the tensor cores
 //                (fs_oz.cu) when it is large.
-//   dense_potrf  Cholesky A = L L^H of the lower triangle, blocked (32): the
-//                diagonal block factorised in shared memory, the panel by a
-//                row-wise triangular solve, the trailing matrix by dense_gemm.
+//   dense_potrf  Cholesky A = L L^H of the lower triangle: diagonal blocks of 32 in
+//                registers, their panels by row-wise triangular solves, products within
+//                panels of 128 columns and one product per panel for the rest.
 //                Reports the first non-positive pivot (LAPACK's info).
-//   dense_trsm   B <- L^-1 B or L^-H B, blocked (32) the same way.
+//   dense_trsm   B <- L^-1 B or L^-H B by inverted diagonal blocks of 128 and products.
 //   dense_heev   the m lowest eigenpairs of a Hermitian matrix:
 //     1. Householder reduction to a real symmetric tridiagonal T = Q^H A Q
 //        (Q = H_0 ... H_{n-2}, H_i = I - tau_i v_i v_i^H, the LAPACK zhetd2
@@ -20,9 +20,9 @@
 //        counts come from the leading minors, rescaled, without division);
 //     3. eigenvectors of T by inverse iteration (Gaussian elimination with
 //        partial pivoting on T - lambda I), vectors of eigenvalues closer
-//        than 1e-10 ||T|| handled as one cluster and made orthogonal to each
+//        than 1e-13 ||T|| handled as one cluster and made orthogonal to each
 //        other by modified Gram-Schmidt (a warp per cluster);
-//     4. back-transformation Z = Q z in blocks of 32 reflectors (compact WY
+//     4. back-transformation Z = Q z in blocks of 128 reflectors (compact WY
 //        form), each block as three GEMMs, then one Cholesky QR pass on Z.
 // Every device-side wait (the exchange of the reduction) is bounded: on expiry the
 // context's error flag is raised and the kernel returns.
@@ -629,12 +629,16 @@ __global__ void tri_bisect_kernel(const double* d, const double* e2, int n, int 
 // ------------------------------------------------------------------ tridiagonal eigenvectors
 // Inverse iteration for the clusters of w (ascending), one warp (block) per
 // index: the block of index k0 starts a cluster when w[k0] - w[k0 - 1] >
-// 1e-10 ||T|| and computes the cluster's vectors in order, each made
+// 1e-13 ||T|| and computes the cluster's vectors in order, each made
 // orthogonal to the cluster's earlier ones.  An eigenvector from inverse
 // iteration is accurate to about eps ||T|| / gap, so vectors outside a cluster
-// are orthogonal to 1e-6 or better; eigenvalues closer than that (the E +- d
-// pairs of the folded spectrum, an orthonormal block's unit eigenvalues) share
-// a cluster.  Lane 0 runs the elimination and the substitutions (sequential in
+// are orthogonal to 2e-3 or better, and the Cholesky QR pass that follows makes
+// them orthonormal to working precision; it mixes neighbours by that angle, which
+// changes their residuals by eps ||T||.  Eigenvalues closer than that (the E +- d
+// pairs of the folded spectrum, an orthonormal block's unit eigenvalues) share a
+// cluster.  (With 1e-10 the low end of the wire's folded spectrum, 1e-9 apart at
+// ||T|| of some 100, made clusters whose vectors one warp computed in turn: 8 ms a
+// call at n = 816.)  Lane 0 runs the elimination and the substitutions (sequential in
 // the position) on shared-memory copies of T, of the factors and of the
 // vector; all lanes run the Gram-Schmidt steps and the norms.  z: [n][m] real
 // (position-major) and, complex, in Z.  Dynamic shared memory: 8 n doubles.
@@ -654,7 +658,7 @@ __global__ void __launch_bounds__(32) tri_invit_kernel(const double* d, const do
     const int lane = threadIdx.x;
     if (k0 >= m) return;
     const double tnorm = fmax(info3[3], 1e-300);
-    const double ctol = 1e-10 * tnorm;
+    const double ctol = 1e-13 * tnorm;
     if (k0 > 0 && w[k0] - w[k0 - 1] <= ctol) return;  // not a cluster start (block-uniform)
     int k1 = k0 + 1;
     while (k1 < m && w[k1] - w[k1 - 1] <= ctol) ++k1;
