@@ -38,6 +38,7 @@ namespace {
 constexpr int TB = 16;       // GEMM tile
 constexpr int TK = 16;       // GEMM k step
 constexpr int NBLK = 32;     // block size of the blocked factorisations
+constexpr int PD_THREADS = 544;  // the 528 elements of a 32 x 32 lower triangle, whole warps
 constexpr long long BAR_LIMIT = 1ll << 22;  // polls of a wait before it gives up
 constexpr int HETRD_SMEM = 224 * 1024;
 
@@ -115,20 +116,26 @@ __global__ void __launch_bounds__(TB * TB) zgemm_kernel(int M, int N, int K, dou
 // ------------------------------------------------------------------ Cholesky
 // Factor the b x b diagonal block at A + j0 (1 + lda); squared pivots to piv[j0 + j]; the
 // first non-positive pivot sets *info = j0 + j + 1 (once) and is replaced by 1 so that the
-// arithmetic stays finite.  Thread (lane r, warp c) keeps element (r, c) in a register; warp j
-// scales column j and hands it over in shared memory, one barrier per column (the chain of a
-// column: reciprocal square root, scaling, barrier, rank-1 term; with the pivot on one thread
-// and three barriers a block took 40 us).
-__global__ void __launch_bounds__(NBLK * NBLK) potrf_diag_kernel(double2* A, int lda, int j0, int b, double* piv,
-                                                                 int* info) {
-    __shared__ double2 col[2][NBLK];
-    const int r = threadIdx.x & (NBLK - 1), c = threadIdx.x >> 5;  // 1024 threads
+// arithmetic stays finite.  A thread keeps one element of the lower triangle in a register, in
+// column order, so that the rank-1 term of column j runs on the warps behind it only (a warp's
+// FP64 instruction costs the same with one lane as with 32: a square of 32 warps spent three
+// times as many: two factorisations at n = 816 3.0 -> 2.2 ms, n = 108 0.35 -> 0.25 ms).  Chain of a column: rank-1 term, hand-over, reciprocal square root, scaling,
+// hand-over.
+__global__ void __launch_bounds__(PD_THREADS) potrf_diag_kernel(double2* A, int lda, int j0, int b, double* piv,
+                                                                int* info) {
+    __shared__ double2 raw[2][NBLK], col[2][NBLK];  // column j before and after scaling
+    // element t of the triangle: column c holds rows c .. 31
+    int r = threadIdx.x, c = 0;
+    while (c < NBLK && r >= NBLK - c) r -= NBLK - c++;
+    r += c;
     double2* D = A + j0 + (long)j0 * lda;
-    double2 a = make_double2(0.0, 0.0);
-    if (r < b && c < b && r >= c) a = D[r + (long)c * lda];
+    const bool live = c < b && r < b;
+    double2 a = live ? D[r + (long)c * lda] : make_double2(0.0, 0.0);
+    if (c == 0) raw[0][r] = a;
+    __syncthreads();
     for (int j = 0; j < b; ++j) {
         if (c == j) {
-            double p = __shfl_sync(0xffffffffu, a.x, j);
+            double p = raw[j & 1][j].x;
             const bool bad = !(p > 0.0);
             if (r == j) {
                 if (piv) piv[j0 + j] = p;
@@ -140,13 +147,15 @@ __global__ void __launch_bounds__(NBLK * NBLK) potrf_diag_kernel(double2* A, int
             col[j & 1][r] = a;
         }
         __syncthreads();
-        if (c > j && r >= c) {
+        if (c > j && c < NBLK) {
             const double2 x = col[j & 1][r], y = col[j & 1][c];  // a -= x conj(y)
             a.x = fma(-x.x, y.x, fma(-x.y, y.y, a.x));
             a.y = fma(x.x, y.y, fma(-x.y, y.x, a.y));
+            if (c == j + 1) raw[c & 1][r] = a;
         }
+        __syncthreads();
     }
-    if (r < b && c < b && r >= c) D[r + (long)c * lda] = a;
+    if (live) D[r + (long)c * lda] = a;
 }
 
 // rows r >= j0 + b of the panel: A[r, j0:j0+b] <- A[r, j0:j0+b] L^-H (L the
@@ -895,7 +904,7 @@ static void potrf_async(fs_ctx* c, int n, double2* A, int lda, double* piv, int*
         const int pe = std::min(n, p0 + PB);
         for (int j0 = p0; j0 < pe; j0 += NBLK) {
             const int b = std::min(NBLK, pe - j0);
-            potrf_diag_kernel<<<1, NBLK * NBLK, 0, c->stream>>>(A, lda, j0, b, piv, info);
+            potrf_diag_kernel<<<1, PD_THREADS, 0, c->stream>>>(A, lda, j0, b, piv, info);
             const int rest = n - j0 - b;
             if (rest <= 0) continue;
             potrf_panel_kernel<<<cdiv((long)rest * 32, 128), 128, 0, c->stream>>>(A, lda, n, j0, b);

@@ -41,6 +41,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 namespace {
 
@@ -758,7 +759,11 @@ void tc_run(fs_ctx* c, int M, int N, int K, const OpA& a, int acont, int amaxk, 
     } else if (!onea) {
         tc_row_max(c, a, acont, M, amaxk, ma);
     }
-    if (!oneb) tc_row_max(c, b, bcont, N, K, mb);
+    if constexpr (std::is_same_v<OpA, LdF2> && std::is_same_v<OpB, LdF2>) {
+        // the Gram matrix of one set of rows: one set of maxima
+        if (!oneb && !onea && !keep && a.rp && a.rp == b.rp && M == N) mb = ma;
+    }
+    if (!oneb && mb != ma) tc_row_max(c, b, bcont, N, K, mb);
     // per-call images in chunks of at most FS_FMT_CHUNK_BYTES: along k for a split result, along
     // the rows of a otherwise
     int kch = nkb, ich = itiles;
