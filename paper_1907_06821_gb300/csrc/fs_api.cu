@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 namespace {
@@ -207,6 +208,60 @@ void ctx_ensure_fp32(fs_ctx* c) { ensure_fp32_tables(c); }
 
 int* ctx_errflag(fs_ctx* c) { return c->errflag_dev; }
 
+// Error flags of the process's contexts: slots of pinned, mapped host pages (pinning a page takes
+// 0.2 ms, so a context does not pin its own).  A page is made when no slot is free and given back
+// when its last slot is; safe from several threads.
+namespace {
+constexpr int FLAG_SLOTS = 256, FLAG_STRIDE = 4;  // 16 bytes apart
+struct FlagPage {
+    int* host = nullptr;
+    int used = 0;
+    bool taken[FLAG_SLOTS] = {};
+};
+std::mutex g_flag_mu;
+std::vector<FlagPage*> g_flag_pages;
+
+int* flag_take() {
+    std::lock_guard<std::mutex> lock(g_flag_mu);
+    FlagPage* pg = nullptr;
+    for (FlagPage* q : g_flag_pages)
+        if (q->used < FLAG_SLOTS) pg = q;
+    if (!pg) {
+        pg = new FlagPage;
+        const cudaError_t e = cudaHostAlloc((void**)&pg->host, FLAG_SLOTS * FLAG_STRIDE * sizeof(int),
+                                            cudaHostAllocMapped | cudaHostAllocPortable);
+        if (e != cudaSuccess) {
+            delete pg;
+            (void)cudaGetLastError();
+            throw fs_error(FS_ERR_OOM, "pinned host allocation failed");
+        }
+        g_flag_pages.push_back(pg);
+    }
+    int i = 0;
+    while (pg->taken[i]) ++i;
+    pg->taken[i] = true;
+    ++pg->used;
+    int* f = pg->host + i * FLAG_STRIDE;
+    *f = 0;
+    return f;
+}
+
+void flag_give(int* f) {
+    std::lock_guard<std::mutex> lock(g_flag_mu);
+    for (size_t q = 0; q < g_flag_pages.size(); ++q) {
+        FlagPage* pg = g_flag_pages[q];
+        if (f < pg->host || f >= pg->host + FLAG_SLOTS * FLAG_STRIDE) continue;
+        pg->taken[(f - pg->host) / FLAG_STRIDE] = false;
+        if (--pg->used == 0) {
+            cudaFreeHost(pg->host);
+            delete pg;
+            g_flag_pages.erase(g_flag_pages.begin() + q);
+        }
+        return;
+    }
+}
+}  // namespace
+
 // wait for the stream and raise FS_ERR_TIMEOUT if a device-side bounded wait gave up (clears
 // the flag, which lives in mapped host memory: reading it costs no copy)
 void ctx_check_errflag(fs_ctx* c) {
@@ -247,8 +302,7 @@ fs_status fs_create(const fs_grid* grid, double ecut, const double k[3], const d
             throw fs_error(FS_ERR_ARG, "bad gemm_path");
         c->gemm_path = c->opt.gemm_path;
         FS_CUDA(cudaGetDevice(&c->device));
-        FS_CUDA(cudaHostAlloc((void**)&c->errflag, sizeof(int), cudaHostAllocMapped));
-        *c->errflag = 0;
+        c->errflag = flag_take();
         FS_CUDA(cudaHostGetDevicePointer((void**)&c->errflag_dev, c->errflag, 0));
         if (c->opt.cuda_stream) {
             c->stream = (cudaStream_t)c->opt.cuda_stream;
@@ -366,7 +420,7 @@ void fs_destroy(fs_ctx* c) {
     prof_release(c);
     cudaStream_t s = c->stream;
     bool own = c->own_stream;
-    if (c->errflag) cudaFreeHost(c->errflag);
+    if (c->errflag) flag_give(c->errflag);
     delete c;
     if (own && s) cudaStreamDestroy(s);
 }
