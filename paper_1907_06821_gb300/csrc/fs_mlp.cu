@@ -428,12 +428,13 @@ __global__ void __launch_bounds__(GT, 1) mlp_grad_kernel(const float* __restrict
     float* lo = hi + NPAD;
     __syncthreads();
     bool first = true;
-    for (int row0 = blockIdx.x * GR; row0 < rows; row0 += gridDim.x * GR, first = false) {
+    // (64-bit rows: a step beyond the last tile passes 2^31 when the row count is near it)
+    for (long row0 = (long)blockIdx.x * GR; row0 < rows; row0 += (long)gridDim.x * GR, first = false) {
         // layer 1: unit j1, half of the rows
         for (int r = hf * (GR / 2); r < (hf + 1) * (GR / 2); ++r) {
             float a = b1;
             if (row0 + r < rows) {
-                const float* f = F + (long)(row0 + r) * 4;
+                const float* f = F + (row0 + r) * 4;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) a += w1[k] * f[k];
             }
@@ -461,7 +462,7 @@ __global__ void __launch_bounds__(GT, 1) mlp_grad_kernel(const float* __restrict
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-            const int row = row0 + 8 * wp + r;
+            const long row = row0 + 8 * wp + r;
             float e = 0.f, w = 0.f;
             if (row < rows) {
                 e = b4 + z - zt[row];
@@ -531,7 +532,7 @@ __global__ void __launch_bounds__(GT, 1) mlp_grad_kernel(const float* __restrict
                     const float dl = h1[r * H + t];
                     sb += dl;
                     if (row0 + r < rows) {
-                        const float* f = F + (long)(row0 + r) * 4;
+                        const float* f = F + (row0 + r) * 4;
 #pragma unroll
                         for (int k = 0; k < 4; ++k) s4[k] = fmaf(dl, f[k], s4[k]);
                     }
@@ -562,7 +563,7 @@ __global__ void sum_parts_kernel(const float* __restrict__ part, int nblk, int n
 __global__ void __launch_bounds__(1024) weight_sum_kernel(const float* __restrict__ w, int n, double* __restrict__ out) {
     __shared__ double sh[32];
     double s = 0;
-    for (int i = threadIdx.x; i < n; i += 8 * 1024) {
+    for (long i = threadIdx.x; i < n; i += 8 * 1024) {
         float v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) v[u] = i + 1024 * u < n ? w[i + 1024 * u] : 0.f;
@@ -817,7 +818,7 @@ double mlp_loss_grad(fs_ctx* c, const float* F, const float* zt, const float* wt
     int dev = 0, nsm = 0;
     FS_CUDA(cudaGetDevice(&dev));
     FS_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int nblk = std::max(1, std::min((rows + GR - 1) / GR, nsm));
+    const int nblk = (int)std::max(1l, std::min(((long)rows + GR - 1) / GR, (long)nsm));
     L.gpart.ensure((size_t)nblk * 2 * NPAD * sizeof(float));
     mlp_grad_kernel<<<nblk, GT, G_SMEM, c->stream>>>(L.P.as<float>(), F, zt, wt, rows, (float)(1.0 / sw),
                                                      L.gpart.as<float>());
