@@ -703,7 +703,7 @@ __global__ void __launch_bounds__(32) tri_invit_kernel(const double* d, const do
                     p2 = 0.0;
                 }
             }
-            ri[n - 1] = p0 == 0.0 ? sep : p0;
+            ri[n - 1] = p0;
             // start vector: a fixed pseudo-random sequence per index
             unsigned int st = 2654435761u * (unsigned int)(k + 1) + 12345u;
             for (int i = 0; i < n; ++i) {
@@ -712,11 +712,15 @@ __global__ void __launch_bounds__(32) tri_invit_kernel(const double* d, const do
             }
         }
         __syncwarp();
-        // small pivots raised to eps ||T||, then their reciprocals (a division per position and
-        // sweep on lane 0 alone would be the longest chain of the iteration)
+        // small pivots raised to 10 eps ||T||, then their reciprocals (a division per position and
+        // sweep on lane 0 alone would be the longest chain of the iteration).  The last pivot is small
+        // whenever lam is an eigenvalue, and raising it by s makes the iteration converge to a
+        // vector of T + s e_n e_n^T: it is only kept above 2^-10 of that (n = 8: residual 1.2e-15
+        // with the last one raised like the others)
         for (int i = lane; i < n; i += 32) {
+            const double least = i < n - 1 ? sep : sep * 0x1p-10;
             double u = ri[i];
-            if (fabs(u) < sep) u = u < 0 ? -sep : sep;
+            if (fabs(u) < least) u = u < 0 ? -least : least;
             ri[i] = 1.0 / u;
         }
         __syncwarp();
