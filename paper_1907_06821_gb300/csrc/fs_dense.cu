@@ -266,6 +266,33 @@ __global__ void hermitize_kernel(double2* A, int n) {
     if (r == c) A[r + (long)c * n].y = 0.0;
 }
 
+// ------------------------------------------------------------------ scaling
+// Powers of two s_i = 2^e with B_ii / 4^e in [0.5, 2) (1 where the diagonal is not a positive
+// number) and their reciprocals: with A and B divided by s_i s_j the factor L of B has rows of
+// norm about one.  The products of a triangular solve are exact only to 2^-55 of (largest of a row)
+// x (largest of a column) on the tensor cores, and rows of B that differ by d make the columns of
+// the inverted blocks and the rows of the right-hand side differ by 1 / d and d: unscaled, a B
+// spread over twelve decades lost four to six digits.  Exact, and no change for a B of unit diagonal.
+__global__ void equil_scale_kernel(const double2* B, int n, double* s) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double b = B[i + (long)i * n].x;
+    const int e = b > 0.0 && isfinite(b) ? (ilogb(b) + 1) >> 1 : 0;
+    s[i] = scalbn(1.0, e);
+    s[n + i] = scalbn(1.0, -e);
+}
+__global__ void equil_sym_kernel(double2* A, double2* B, int n, const double* s) {
+    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (t >= (long)n * n) return;
+    const double fr = s[n + t % n], fc = s[n + t / n];
+    A[t] = cscale(cscale(A[t], fr), fc);
+    B[t] = cscale(cscale(B[t], fr), fc);
+}
+__global__ void equil_rows_kernel(double2* Z, int n, int m, const double* s) {
+    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (t < (long)n * m) Z[t] = cscale(Z[t], s[n + t % n]);
+}
+
 // ------------------------------------------------------------------ tridiagonal reduction
 // Full Hermitian A (n x n, both triangles).  Step i: reflector v_i (v[0] = 1 at
 // row i + 1) with H^H x = beta e_1 for x = A[i+1:, i]; y_i = A22 v_i;
@@ -952,6 +979,8 @@ static void tri_inverses(fs_ctx* c, int n, const double2* L, int lda) {
 // B <- L^-1 B (conj = 0) or L^-H B (conj = 1); L lower n x n (ld lda), B n x ncols (ld ldb).
 // Blocks of IB rows: x_b = inv(L_bb) b_b, then the rest of B minus its product with x_b.
 // fresh = false: the inverses of the last call's L are the ones of this L.
+// The products are as exact as the rows of L are evenly scaled (see equil_scale_kernel): callers
+// pass the factor of a matrix whose diagonal entries are of one size.
 void dense_trsm(fs_ctx* c, int conj, int n, int ncols, const double2* L, int lda, double2* B, int ldb, bool fresh) {
     if (n <= 0 || ncols <= 0) return;
     ProfScope ps(c, KS_SUB_TRSM, 0.0, 4.0 * n * (double)n * ncols);
@@ -1112,12 +1141,17 @@ void dense_heev(fs_ctx* c, int n, double2* A, int m, double* w, double2* Z, int 
 
 // Generalised Hermitian problem GA x = lambda GB x (both n x n, ld n; GB positive
 // definite): the m lowest pairs; eigenvectors (GB-orthonormal) overwrite GA's
-// first m columns, eigenvalues to w.  GB is overwritten by its Cholesky factor.
+// first m columns, eigenvalues to w.  GB is overwritten (the Cholesky factor of the scaled GB).
 // Returns the Cholesky info (0 = success).
 int dense_hegv(fs_ctx* c, int n, double2* GA, double2* GB, int m, double* w) {
+    DenseWork& D = c->dense;
+    D.equil.ensure((size_t)2 * n * sizeof(double));
+    const double* s = D.equil.as<double>();
+    equil_scale_kernel<<<cdiv(n, 256), 256, 0, c->stream>>>(GB, n, D.equil.as<double>());
+    equil_sym_kernel<<<cdiv((long)n * n, 256), 256, 0, c->stream>>>(GA, GB, n, s);
+    FS_CUDA(cudaGetLastError());
     int info = dense_potrf(c, n, GB, n, nullptr);
     if (info != 0) return info;
-    DenseWork& D = c->dense;
     D.T.ensure((size_t)n * n * sizeof(double2));
     D.U.ensure((size_t)n * m * sizeof(double2));
     double2* T = D.T.as<double2>();
@@ -1127,6 +1161,8 @@ int dense_hegv(fs_ctx* c, int n, double2* GA, double2* GB, int m, double* w) {
     dense_trsm(c, 0, n, n, GB, n, T, n, false);        // L^-1 GA L^-H
     dense_heev(c, n, T, m, w, D.U.as<double2>(), n);
     dense_trsm(c, 1, n, m, GB, n, D.U.as<double2>(), n, true);  // x = L^-H y
+    equil_rows_kernel<<<cdiv((long)n * m, 256), 256, 0, c->stream>>>(D.U.as<double2>(), n, m, s);
+    FS_CUDA(cudaGetLastError());
     FS_CUDA(cudaMemcpyAsync(GA, D.U.p, (size_t)n * m * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
     return 0;
 }

@@ -13,10 +13,13 @@
 // read out as integers and added to two 64-bit integers per output,
 //     hi += D_0 2^16 + D_1 2^8 + D_2,   lo += D_3 2^24 + D_4 2^16 + D_5 2^8 + D_6 + D_7 / 2^8
 // (the last rounded to an integer), and C = (hi 2^32 + lo) 2^(Ea + Eb - 62).
-// The error is that of the cut (2^-56 of the row maximum per component); the digit
-// pairs left out (i + j > 7) and the rounding of D_7 are below it.  Without the
-// pairs i + j = 7 (28 MMAs a stage instead of 34) the error was 1.5 to 8 times that
-// of an FP64 FMA chain; with them it is no larger.
+// The error is that of the cut, up to 2^-55 of the row maximum per component (2^(E - 56), and
+// the maximum may be 2^(E - 1)); the digit pairs left out (i + j > 7) and the rounding of D_7 are
+// below it.  So it is relative to (largest |a| of a row) x (largest |b| of a column), where an FMA
+// chain's is relative to sum |a||b|: no larger for operands whose k contribute alike (Gram
+// products, rotations, projections; with 28 MMAs a stage, without the pairs i + j = 7, it was 1.5
+// to 8 times as large), larger where a and b are graded along k in opposite directions.  The
+// triangular solves, where that can happen, work on scaled factors (fs_dense.cu).
 //
 // Why: GB300 does about 2 FP64 FMAs per clock and SM (0.65 TFLOP/s through a GEMM);
 // 34 BF16 digit products at the tensor rate are some 50 times as fast.  What bounds

@@ -1,4 +1,5 @@
-"""Accuracy of the dense eigensolver where the way it computes shows: small matrices."""
+"""Accuracy of the dense eigensolver where the way it computes shows: small matrices, and rows
+of very different size."""
 import numpy as np
 import pytest
 
@@ -47,3 +48,44 @@ def test_multiples_of_the_unit_matrix(ctx):
         w, Z = ctx.dense_eigh(3.0 * np.eye(n, dtype=complex), m=n)
         assert np.abs(w - 3.0).max() < 8 * U * 3.0
         assert np.abs(Z.conj().T @ Z - np.eye(n)).max() < 64 * n * U
+
+
+# n = 600 and 816 take the triangular solves' products to the tensor cores; D runs up, down or
+# mixed over six (1e-6 .. 1) or twelve decades (1e-6 .. 1e6)
+@pytest.mark.parametrize("n,lo,hi", [(600, -6, 6), (816, -6, 0)])
+@pytest.mark.parametrize("order", ["up", "down", "mixed"])
+def test_graded_b(ctx, n, lo, hi, order):
+    """A = D A' D, B = D B' D: the eigenvalues are those of (A', B') and Y = D Z is B'-orthonormal.
+    Cholesky and triangular substitution are indifferent to D, so the tolerance is that of the
+    evenly scaled problem, 64 n u, of which the measured values are a few tenths of a percent: a
+    hundredth of it, 0.64 n u, is asked for."""
+    rng = np.random.default_rng(n)
+    m = n // 3
+    A, B = _herm(rng, n), np.eye(n) + 0.3 * _herm(rng, n)
+    D = 10.0 ** np.linspace(lo, hi, n)
+    D = {"up": D, "down": D[::-1], "mixed": rng.permutation(D)}[order]
+    Ad, Bd = D[:, None] * A * D, D[:, None] * B * D
+    A = ((Ad + Ad.conj().T) / 2) / D[:, None] / D
+    B = ((Bd + Bd.conj().T) / 2) / D[:, None] / D
+    w, Z = ctx.dense_eigh((Ad + Ad.conj().T) / 2, m=m, B=(Bd + Bd.conj().T) / 2)
+    Y = D[:, None] * Z
+    tol = 0.64 * n * U
+    assert np.abs(Y.conj().T @ B @ Y - np.eye(m)).max() < tol
+    assert np.abs(A @ Y - B @ Y * w).max() < tol
+
+
+def test_scaled_and_indefinite_b(ctx):
+    """B of any size by an exact power of two gives the same vectors; a B that is not positive
+    definite is reported by its column, also with zeros and negative numbers on the diagonal."""
+    from paper_1907_06821_gb300 import FSError, FS_ERR_NUMERIC
+    rng = np.random.default_rng(5)
+    A, B = _herm(rng, 48), np.eye(48) + 0.3 * _herm(rng, 48)
+    w, Z = ctx.dense_eigh(A, m=48, B=B)
+    w2, Z2 = ctx.dense_eigh(A, m=48, B=B * 2.0 ** -200)
+    assert np.array_equal(w * 2.0 ** 200, w2) and np.array_equal(Z * 2.0 ** 100, Z2)
+    for v in (0.0, -1.0, np.nan):
+        C = B.copy()
+        C[20, 20] = v
+        with pytest.raises(FSError, match="column") as ei:
+            ctx.dense_eigh(A, m=4, B=C)
+        assert ei.value.code == FS_ERR_NUMERIC
