@@ -372,8 +372,11 @@ fs_status fs_dense_eigh(fs_ctx* ctx, int n, const void* A, const void* B, int m,
 /* Failure-path check without a GPU fault: runs the library's bounded device wait (the one
  * the tensor-core pipelines use) on a barrier that nothing completes, polling `polls`
  * times (1 .. 2^24); the wait gives up, raises the context's error flag, and the call
- * returns FS_ERR_TIMEOUT as a pipeline timeout would.  The context stays usable. */
+ * returns FS_ERR_TIMEOUT as a pipeline timeout would.  The context stays usable.
+ * The second form starts the same wait and returns: the next call on the context, whatever it
+ * computes, reports the timeout. */
 fs_status fs_wait_selftest(fs_ctx* ctx, long long polls);
+fs_status fs_wait_selftest_pending(fs_ctx* ctx, long long polls);
 
 /* Release everything the context holds.  NULL is accepted. */
 void fs_destroy(fs_ctx* ctx);

@@ -138,6 +138,8 @@ def load_library(path: str = LIB_PATH):
     lib.fs_dense_eigh.restype = ip
     lib.fs_wait_selftest.argtypes = [vp, C.c_longlong]
     lib.fs_wait_selftest.restype = ip
+    lib.fs_wait_selftest_pending.argtypes = [vp, C.c_longlong]
+    lib.fs_wait_selftest_pending.restype = ip
     lib.fs_autotune.argtypes = [vp, C.POINTER(C.c_int)]
     lib.fs_autotune.restype = ip
     lib.fs_profile.argtypes = [vp, ip]
@@ -382,10 +384,12 @@ class Context:
                                            _dptr(w), Z.ctypes.data), "fs_dense_eigh")
         return w, Z
 
-    def wait_selftest(self, polls=4096):
+    def wait_selftest(self, polls=4096, pending=False):
         """Run the bounded device wait on a barrier nothing completes; raises FSError
-        with FS_ERR_TIMEOUT (the failure path of the tensor-core pipelines)."""
-        self._check(self.lib.fs_wait_selftest(self.h, int(polls)), "fs_wait_selftest")
+        with FS_ERR_TIMEOUT (the failure path of the tensor-core pipelines).  pending:
+        only start it, so that the next call raises."""
+        call = self.lib.fs_wait_selftest_pending if pending else self.lib.fs_wait_selftest
+        self._check(call(self.h, int(polls)), "fs_wait_selftest")
 
     # ------------------------------------------------ ChebFD
     def spectral_bounds(self, iters=40):

@@ -42,20 +42,6 @@ __global__ void beta_kernel(double2* __restrict__ beta, const int* __restrict__ 
     }
 }
 
-template <typename Fn> fs_status guarded(fs_ctx* c, Fn fn) {
-    try {
-        fn();
-        if (c) c->err.clear();
-        return FS_OK;
-    } catch (const fs_error& e) {
-        if (c) c->err = e.msg;
-        return e.code;
-    } catch (const std::bad_alloc&) {
-        if (c) c->err = "host allocation failed";
-        return FS_ERR_OOM;
-    }
-}
-
 int posmod(long a, int n) { return (int)(((a % n) + n) % n); }
 
 void build_sphere(fs_ctx* c) {
@@ -264,12 +250,24 @@ void flag_give(int* f) {
 
 // wait for the stream and raise FS_ERR_TIMEOUT if a device-side bounded wait gave up (clears
 // the flag, which lives in mapped host memory: reading it costs no copy)
+static bool take_errflag(fs_ctx* c) {
+    if (!*(volatile int*)c->errflag) return false;
+    *(volatile int*)c->errflag = 0;
+    return true;
+}
+static const char* TIMEOUT_MSG = "a tensor-core pipeline wait exceeded its limit";
 void ctx_check_errflag(fs_ctx* c) {
     FS_CUDA(cudaStreamSynchronize(c->stream));
-    if (*(volatile int*)c->errflag) {
-        *(volatile int*)c->errflag = 0;
-        throw fs_error(FS_ERR_TIMEOUT, "a tensor-core pipeline wait exceeded its limit");
+    if (take_errflag(c)) throw fs_error(FS_ERR_TIMEOUT, TIMEOUT_MSG);
+}
+
+fs_status ctx_fail(fs_ctx* c, fs_status code, const std::string& msg) {
+    if (c->errflag && c->stream && cudaStreamSynchronize(c->stream) == cudaSuccess && take_errflag(c)) {
+        c->err = TIMEOUT_MSG;
+        return FS_ERR_TIMEOUT;
     }
+    c->err = msg;
+    return code;
 }
 
 extern "C" {
@@ -284,7 +282,7 @@ fs_status fs_create(const fs_grid* grid, double ecut, const double k[3], const d
     if (!(ecut > 0) || !std::isfinite(ecut)) return FS_ERR_ARG;
     fs_ctx* c = new (std::nothrow) fs_ctx();
     if (!c) return FS_ERR_OOM;
-    fs_status st = guarded(c, [&] {
+    fs_status st = ctx_call(c, [&] {
         std::memcpy(c->L, grid->L, sizeof(c->L));
         std::memcpy(c->n, grid->n, sizeof(c->n));
         std::memcpy(c->k, k, sizeof(c->k));
@@ -347,7 +345,7 @@ fs_status fs_apply_H(fs_ctx* c, const void* psi, void* hpsi, int nband, double s
         c->err = "fs_apply_H: bad precision";
         return FS_ERR_ARG;
     }
-    return guarded(c, [&] {
+    return ctx_call(c, [&] {
         if (nband == 0) return;
         if (precision == FS_FP64) {
             apply_H_impl<double2>(c, (const double2*)psi, (double2*)hpsi, nband, shift);
@@ -355,7 +353,6 @@ fs_status fs_apply_H(fs_ctx* c, const void* psi, void* hpsi, int nband, double s
             ensure_fp32_tables(c);
             apply_H_impl<float2>(c, (const float2*)psi, (float2*)hpsi, nband, shift);
         }
-        ctx_check_errflag(c);  // (waits for the stream)
     });
 }
 
@@ -365,7 +362,7 @@ fs_status fs_set_initial_states(fs_ctx* c, const void* psi, int n, int damp, int
         c->err = "fs_set_initial_states: bad arguments";
         return FS_ERR_ARG;
     }
-    return guarded(c, [&] {
+    return ctx_call(c, [&] {
         c->ninit = n;
         c->init_damp = damp ? 1 : 0;
         if (n == 0) return;
@@ -384,7 +381,7 @@ fs_status fs_solve(fs_ctx* c, double e_ref, int nstates, double tol, fs_result* 
         return FS_ERR_ARG;
     }
     fs_status st = FS_OK;
-    fs_status g = guarded(c, [&] { st = solve_impl(c, e_ref, nstates, tol, res); });
+    fs_status g = ctx_call(c, [&] { st = solve_impl(c, e_ref, nstates, tol, res); });
     return g != FS_OK ? g : st;
 }
 
@@ -395,7 +392,7 @@ fs_status fs_solve_lowest(fs_ctx* c, int nstates, double tol, fs_result* res) {
         return FS_ERR_ARG;
     }
     fs_status st = FS_OK;
-    fs_status g = guarded(c, [&] { st = solve_impl(c, 0.0, nstates, tol, res, true); });
+    fs_status g = ctx_call(c, [&] { st = solve_impl(c, 0.0, nstates, tol, res, true); });
     return g != FS_OK ? g : st;
 }
 
@@ -405,7 +402,7 @@ fs_status fs_get_states(fs_ctx* c, void* psi, int n, int where) {
         c->err = "fs_get_states: bad arguments (n exceeds the states of the last solve?)";
         return FS_ERR_ARG;
     }
-    return guarded(c, [&] {
+    return ctx_call(c, [&] {
         if (n == 0) return;
         size_t bytes = (size_t)n * c->npw * sizeof(double2);
         FS_CUDA(cudaMemcpyAsync(psi, c->result_states.p, bytes,

@@ -46,6 +46,7 @@ template <typename T2> double time_apply(fs_ctx* c, int nb, int reps) {
     cudaEventElapsedTime(&ms, a, b);
     cudaEventDestroy(a);
     cudaEventDestroy(b);
+    ctx_check_errflag(c);
     return ms;
 }
 }  // namespace
@@ -59,7 +60,7 @@ extern "C" {
 // and precision for the process.  verbose > 0 prints each timing on stderr.
 fs_status fs_autotune(fs_ctx* c, int* cpb_out) {
     if (!c) return FS_ERR_ARG;
-    try {
+    return ctx_call(c, [&] {
         const bool fp32 = c->opt.precision == FS_MIXED;
         auto key = std::make_tuple(c->n[0], c->n[1], c->n[2], c->ncol, (int)fp32);
         {
@@ -70,7 +71,7 @@ fs_status fs_autotune(fs_ctx* c, int* cpb_out) {
                 c->pf_ipt = it->second.ipt;
                 c->hchunk_bytes = it->second.chunk;
                 if (cpb_out) *cpb_out = c->cpb;
-                return FS_OK;
+                return;
             }
         }
         const int nb = 32;
@@ -123,12 +124,7 @@ fs_status fs_autotune(fs_ctx* c, int* cpb_out) {
             g_tuned[key] = Tuned{c->cpb, c->pf_ipt, c->hchunk_bytes};
         }
         if (cpb_out) *cpb_out = c->cpb;
-        c->err.clear();
-        return FS_OK;
-    } catch (const fs_error& e) {
-        c->err = e.msg;
-        return e.code;
-    }
+    });
 }
 
 fs_status fs_batch_create(int nbox, fs_ctx* const* ctxs, int nthreads, fs_batch** out) {

@@ -324,17 +324,7 @@ fs_status fs_spectral_bounds(fs_ctx* c, int iters, double* emin, double* emax) {
         c->err = "fs_spectral_bounds: bad arguments";
         return FS_ERR_ARG;
     }
-    try {
-        spectral_bounds_impl(c, iters, emin, emax);
-        c->err.clear();
-        return FS_OK;
-    } catch (const fs_error& e) {
-        c->err = e.msg;
-        return e.code;
-    } catch (const std::bad_alloc&) {
-        c->err = "host allocation failed";
-        return FS_ERR_OOM;
-    }
+    return ctx_call(c, [&] { spectral_bounds_impl(c, iters, emin, emax); });
 }
 
 fs_status fs_chebfd(fs_ctx* c, double e_ref, double half_width, double emin, double emax, int degree, int nvec,
@@ -346,17 +336,10 @@ fs_status fs_chebfd(fs_ctx* c, double e_ref, double half_width, double emin, dou
         c->err = "fs_chebfd: bad arguments";
         return FS_ERR_ARG;
     }
-    try {
-        fs_status st = chebfd_impl(c, e_ref, half_width, emin, emax, degree, nvec, steps, seed, nwant, res);
-        c->err.clear();
-        return st;
-    } catch (const fs_error& e) {
-        c->err = e.msg;
-        return e.code;
-    } catch (const std::bad_alloc&) {
-        c->err = "host allocation failed";
-        return FS_ERR_OOM;
-    }
+    fs_status st = FS_OK;
+    const fs_status g =
+        ctx_call(c, [&] { st = chebfd_impl(c, e_ref, half_width, emin, emax, degree, nvec, steps, seed, nwant, res); });
+    return g != FS_OK ? g : st;
 }
 
 }  // extern "C"

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -407,6 +408,22 @@ template <typename T2> void beta_project_chunked(fs_ctx* c, const T2* psi, const
 template <typename T2> void beta_add_chunked(fs_ctx* c, const double2* Q, int nb, T2* hpsi);
 int* ctx_errflag(fs_ctx* c);
 void ctx_check_errflag(fs_ctx* c);
+// Body of an entry point: its errors as a status and a message.  A device-side wait that gave up
+// leaves numbers that are not results, so every call reads the error flag before it returns, and a
+// failure with the flag raised is reported as the timeout that it follows from.
+fs_status ctx_fail(fs_ctx* c, fs_status code, const std::string& msg);
+template <typename Fn> fs_status ctx_call(fs_ctx* c, Fn fn) {
+    try {
+        fn();
+        ctx_check_errflag(c);
+        c->err.clear();
+        return FS_OK;
+    } catch (const fs_error& e) {
+        return ctx_fail(c, e.code, e.msg);
+    } catch (const std::bad_alloc&) {
+        return ctx_fail(c, FS_ERR_OOM, "host allocation failed");
+    }
+}
 
 // vector kernels (fs_vec.cu)
 template <typename T2>

@@ -964,7 +964,7 @@ int dense_potrf(fs_ctx* c, int n, double2* A, int lda, double* piv) {
     potrf_async(c, n, A, lda, piv, D.info.as<int>());
     int h = 0;
     FS_CUDA(cudaMemcpyAsync(&h, D.info.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    FS_CUDA(cudaStreamSynchronize(c->stream));
+    ctx_check_errflag(c);  // (synchronises; before the info of a product that gave up is taken for one)
     return h;
 }
 
@@ -1174,7 +1174,7 @@ extern "C" fs_status fs_dense_eigh(fs_ctx* c, int n, const void* A, const void* 
         c->err = "fs_dense_eigh: bad arguments";
         return FS_ERR_ARG;
     }
-    try {
+    return ctx_call(c, [&] {
         const size_t bytes = (size_t)n * n * sizeof(double2);
         dbuf dA, dB, dZ, dw;
         dA.alloc(bytes);
@@ -1195,11 +1195,5 @@ extern "C" fs_status fs_dense_eigh(fs_ctx* c, int n, const void* A, const void* 
         FS_CUDA(cudaMemcpyAsync(w, dw.p, (size_t)m * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         FS_CUDA(cudaMemcpyAsync(Z, dZ.p, (size_t)n * m * sizeof(double2), cudaMemcpyDeviceToHost, c->stream));
         FS_CUDA(cudaStreamSynchronize(c->stream));
-        ctx_check_errflag(c);
-        c->err.clear();
-        return FS_OK;
-    } catch (const fs_error& e) {
-        c->err = e.msg;
-        return e.code;
-    }
+    });
 }

@@ -55,7 +55,7 @@ extern "C" fs_status fs_kinterp(fs_ctx* c, double alpha, int n1, const double* e
         c->err = "fs_kinterp: bad arguments (need 0 < n1 <= n2, n1 <= 2048)";
         return FS_ERR_ARG;
     }
-    try {
+    return ctx_call(c, [&] {
         const long N = c->npw;
         const double2* P1 = static_cast<const double2*>(psi1);  // column-major N x n1 (rows of [n1][npw])
         const double2* P2 = static_cast<const double2*>(psi2);
@@ -95,11 +95,5 @@ extern "C" fs_status fs_kinterp(fs_ctx* c, double alpha, int n1, const double* e
         dense_gemm(c, 0, 0, (int)N, n1, n2, 1.0 - alpha, P2, (int)N, M2.as<double2>(), n2, 1.0, Out, (int)N);
         FS_CUDA(cudaMemcpyAsync(eps, dw.p, n1 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         FS_CUDA(cudaStreamSynchronize(c->stream));
-        ctx_check_errflag(c);
-        c->err.clear();
-        return FS_OK;
-    } catch (const fs_error& e) {
-        c->err = e.msg;
-        return e.code;
-    }
+    });
 }

@@ -326,11 +326,11 @@ fs_status fs_set_linear_states(fs_ctx* c, const void* phi, const double* eps, co
         c->err = "fs_set_linear_states: bad arguments (n beyond the last solve's states?)";
         return FS_ERR_ARG;
     }
-    try {
+    return ctx_call(c, [&] {
         c->lin_n = 0;
         c->lin_eps.clear();
         c->lin_delta.clear();
-        if (n == 0) return FS_OK;
+        if (n == 0) return;
         const size_t bytes = (size_t)n * c->npw * sizeof(double2);
         c->lin_phi.ensure(bytes);
         if (phi) {
@@ -346,15 +346,7 @@ fs_status fs_set_linear_states(fs_ctx* c, const void* phi, const double* eps, co
         }
         FS_CUDA(cudaStreamSynchronize(c->stream));
         c->lin_n = n;
-        c->err.clear();
-        return FS_OK;
-    } catch (const fs_error& e) {
-        c->err = e.msg;
-        return e.code;
-    } catch (const std::bad_alloc&) {
-        c->err = "host allocation failed";
-        return FS_ERR_OOM;
-    }
+    });
 }
 
 fs_status fs_linear_solve(fs_ctx* c, double e_ref, const void* w, void* psi, int nrhs, int where, int from_psi,
@@ -369,7 +361,8 @@ fs_status fs_linear_solve(fs_ctx* c, double e_ref, const void* w, void* psi, int
     res->n_hpsi = 0;
     res->seconds = 0;
     if (nrhs == 0) return FS_OK;
-    try {
+    fs_status st = FS_OK;
+    const fs_status g = ctx_call(c, [&] {
         const size_t vb = (size_t)nrhs * c->npw * sizeof(double2);
         const double2* wd = (const double2*)w;
         double2* pd = (double2*)psi;
@@ -382,20 +375,14 @@ fs_status fs_linear_solve(fs_ctx* c, double e_ref, const void* w, void* psi, int
             wd = c->lin_io[0].as<double2>();
             pd = c->lin_io[1].as<double2>();
         }
-        fs_status st = linear_solve_impl(c, e_ref, wd, pd, nrhs, from_psi != 0, tol, maxit, res);
+        st = linear_solve_impl(c, e_ref, wd, pd, nrhs, from_psi != 0, tol, maxit, res);
         if (where == FS_HOST) {
             FS_CUDA(cudaMemcpyAsync(psi, pd, vb, cudaMemcpyDeviceToHost, c->stream));
             FS_CUDA(cudaStreamSynchronize(c->stream));
         }
-        c->err = st == FS_OK ? "" : "fs_linear_solve: some right-hand side did not reach tol";
-        return st;
-    } catch (const fs_error& e) {
-        c->err = e.msg;
-        return e.code;
-    } catch (const std::bad_alloc&) {
-        c->err = "host allocation failed";
-        return FS_ERR_OOM;
-    }
+    });
+    if (g == FS_OK && st != FS_OK) c->err = "fs_linear_solve: some right-hand side did not reach tol";
+    return g != FS_OK ? g : st;
 }
 
 }  // extern "C"

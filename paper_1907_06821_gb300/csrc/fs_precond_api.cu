@@ -10,17 +10,6 @@
 void ctx_ensure_fp32(fs_ctx* c);
 
 namespace {
-template <typename Fn> fs_status guard(fs_ctx* c, Fn fn) {
-    try {
-        fn();
-        c->err.clear();
-        return FS_OK;
-    } catch (const fs_error& e) {
-        c->err = e.msg;
-        return e.code;
-    }
-}
-
 __global__ void d2f_kernel(const double2* in, float2* out, long n) {
     for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x)
         out[t] = make_float2((float)in[t].x, (float)in[t].y);
@@ -72,7 +61,7 @@ fs_status fs_precond_train(fs_ctx* c, double e_ref, int nstates, double tol, int
         return FS_ERR_ARG;
     }
     const int saved = c->opt.precond;
-    fs_status st = guard(c, [&] {
+    fs_status st = ctx_call(c, [&] {
         mlp_setup(c);
         Mlp& L = c->mlp;
         std::vector<double> eps(nstates), res(nstates);
@@ -130,7 +119,7 @@ fs_status fs_precond_weights(fs_ctx* c, float* w, int n, int set) {
         c->err = "fs_precond_weights: n must be " + std::to_string(mlp_nparam());
         return FS_ERR_ARG;
     }
-    return guard(c, [&] {
+    return ctx_call(c, [&] {
         mlp_setup(c);
         Mlp& L = c->mlp;
         if (set) {
@@ -152,11 +141,9 @@ fs_status fs_precond_eval(fs_ctx* c, const float* features, int rows, float* z) 
         c->err = "fs_precond_eval: bad arguments";
         return FS_ERR_ARG;
     }
-    return guard(c, [&] {
+    return ctx_call(c, [&] {
         mlp_setup(c);
         mlp_forward(c, features, rows, z);
-        FS_CUDA(cudaStreamSynchronize(c->stream));
-        ctx_check_errflag(c);  // a bounded wait of the tensor-core forward that gave up
     });
 }
 
@@ -169,7 +156,7 @@ fs_status fs_precond_features(fs_ctx* c, double e_ref, const void* R, const void
         return FS_ERR_ARG;
     }
     if (nb == 0) return FS_OK;
-    return guard(c, [&] {
+    return ctx_call(c, [&] {
         mlp_setup(c);
         Mlp& L = c->mlp;
         if (L.e_ref != e_ref || !L.Mdev.p) {
@@ -193,7 +180,7 @@ fs_status fs_precond_loss_grad(fs_ctx* c, const float* features, const float* ta
         c->err = "fs_precond_loss_grad: bad arguments";
         return FS_ERR_ARG;
     }
-    return guard(c, [&] {
+    return ctx_call(c, [&] {
         mlp_setup(c);
         // inputs made on the legacy default stream are complete before this stream reads them
         FS_CUDA(cudaStreamSynchronize(cudaStreamLegacy));

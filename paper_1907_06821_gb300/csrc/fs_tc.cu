@@ -905,20 +905,23 @@ template void tc_gemm_nn<double2>(fs_ctx*, int, int, int, const double2*, long, 
 template void tc_gemm_nn<float2>(fs_ctx*, int, int, int, const float2*, long, long, const float2*, long, const int*,
                                  float2*, long, const int*, double, double, const float2*, long, int, const BetaGen*);
 
-extern "C" fs_status fs_wait_selftest(fs_ctx* c, long long polls) {
+namespace {
+fs_status wait_selftest(fs_ctx* c, long long polls, bool pending) {
     if (!c) return FS_ERR_ARG;
     if (polls < 1 || polls > (1ll << 24)) {
         c->err = "fs_wait_selftest: polls out of range [1, 2^24]";
         return FS_ERR_ARG;
     }
-    try {
+    if (pending) {
+        wait_selftest_kernel<<<1, 32, 0, c->stream>>>(polls, ctx_errflag(c));
+        return cudaGetLastError() == cudaSuccess ? FS_OK : FS_ERR_CUDA;
+    }
+    return ctx_call(c, [&] {
         wait_selftest_kernel<<<1, 32, 0, c->stream>>>(polls, ctx_errflag(c));
         FS_CUDA(cudaGetLastError());
-        ctx_check_errflag(c);
-        c->err.clear();
-        return FS_OK;
-    } catch (const fs_error& e) {
-        c->err = e.msg;
-        return e.code;
-    }
+    });
 }
+}  // namespace
+
+extern "C" fs_status fs_wait_selftest(fs_ctx* c, long long polls) { return wait_selftest(c, polls, false); }
+extern "C" fs_status fs_wait_selftest_pending(fs_ctx* c, long long polls) { return wait_selftest(c, polls, true); }
