@@ -554,7 +554,8 @@ __global__ void sum_parts_kernel(const float* __restrict__ part, int nblk, int n
 #pragma unroll 4
     for (int b = 0; b < nblk; ++b) {
         const float* h = part + (size_t)b * 2 * NPAD + p;
-        s += (double)h[0] + (double)h[NPAD];
+        // (where the sum overflowed, the error term is Inf - Inf)
+        s += isfinite(h[0]) ? (double)h[0] + (double)h[NPAD] : (double)h[0];
     }
     out[p] = (float)s;
 }

@@ -1,4 +1,4 @@
-"""The training step at the limits of its inputs: row counts near 2^31."""
+"""The training step at the limits of its inputs: row counts near 2^31, targets without a finite loss."""
 import numpy as np
 import pytest
 
@@ -51,3 +51,22 @@ def test_row_counts_near_2_31(ctx):
     torch.cuda.empty_cache()
     assert abs(loss - loss0) < 64 * 2.0 ** -24 * loss0
     assert (g - g0).abs().max().item() < 64 * 2.0 ** -24 * g0.abs().max().item()
+
+
+@pytest.mark.parametrize("rows", [50, 20000])  # one block; more than one tile per block
+def test_infinite_loss(ctx, rows):
+    """A loss beyond the FP32 range is infinite, not a NaN, and so are the gradients of the output
+    layer for an infinite target (FP32 has them as sums of infinities of one sign)."""
+    F, zt, wt = _rows(4, rows)
+    zt[7] = 3e25
+    torch.cuda.synchronize()
+    assert ctx.precond_loss_grad(F, zt, wt)[0] == float("inf")
+    zt[7] = float("inf")
+    torch.cuda.synchronize()
+    loss, g = ctx.precond_loss_grad(F, zt, wt)
+    assert loss == float("inf")
+    assert g[-1].item() == -float("inf") and torch.isinf(g[-129:]).all()
+    zt[7] = float("nan")
+    torch.cuda.synchronize()
+    loss, g = ctx.precond_loss_grad(F, zt, wt)
+    assert np.isnan(loss) and torch.isnan(g[-129:]).all()
