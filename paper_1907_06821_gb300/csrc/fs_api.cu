@@ -261,6 +261,11 @@ void ctx_check_errflag(fs_ctx* c) {
     if (take_errflag(c)) throw fs_error(FS_ERR_TIMEOUT, TIMEOUT_MSG);
 }
 
+static thread_local fs_ctx* t_ctx = nullptr;
+CtxScope::CtxScope(fs_ctx* c) : outer(t_ctx) { t_ctx = c; }
+CtxScope::~CtxScope() { t_ctx = outer; }
+bool ctx_give_back() { return t_ctx && t_ctx->oz.give_back(); }
+
 fs_status ctx_fail(fs_ctx* c, fs_status code, const std::string& msg) {
     if (c->errflag && c->stream && cudaStreamSynchronize(c->stream) == cudaSuccess && take_errflag(c)) {
         c->err = TIMEOUT_MSG;

@@ -105,19 +105,29 @@ struct fs_error {
 };
 
 // ------------------------------------------------------------------ device buffer
+// Memory that the running call's context holds only to be faster (the FP64 digit images of its
+// projector table) is given back when an allocation fails; true if there was any (fs_api.cu).
+bool ctx_give_back();
+
 struct dbuf {
     void* p = nullptr;
     size_t bytes = 0;
-    void alloc(size_t nb) {
+    bool try_alloc(size_t nb) {
         release();
-        if (nb == 0) return;
-        cudaError_t e = cudaMalloc(&p, nb);
-        if (e != cudaSuccess) {
+        if (nb == 0) return true;
+        do {
+            if (cudaMalloc(&p, nb) == cudaSuccess) {
+                bytes = nb;
+                return true;
+            }
             p = nullptr;
             (void)cudaGetLastError();
-            throw fs_error(FS_ERR_OOM, "cudaMalloc of " + std::to_string(nb) + " bytes failed");
-        }
-        bytes = nb;
+        } while (ctx_give_back());
+        return false;
+    }
+    bool try_ensure(size_t nb) { return nb <= bytes || try_alloc(nb); }
+    void alloc(size_t nb) {
+        if (!try_alloc(nb)) throw fs_error(FS_ERR_OOM, "cudaMalloc of " + std::to_string(nb) + " bytes failed");
     }
     void ensure(size_t nb) {
         if (nb > bytes) alloc(nb);
@@ -238,6 +248,16 @@ struct DenseWork {
 // (kept), per-call images, row maxima and split-K partial sums.
 struct OzWork {
     dbuf table_g, table_n, max_g, max_n, aimg, bimg, ma, mb, part;
+    bool have_g = false, have_n = false;  // the table image is complete
+    bool no_image = false;                // there was no room for one: products go by chunks
+    bool give_back() {
+        const bool any = table_g.p || table_n.p;
+        table_g.release();
+        table_n.release();
+        have_g = have_n = false;
+        no_image = no_image || any;
+        return any;
+    }
 };
 
 struct SolverSmall {
@@ -412,7 +432,14 @@ void ctx_check_errflag(fs_ctx* c);
 // leaves numbers that are not results, so every call reads the error flag before it returns, and a
 // failure with the flag raised is reported as the timeout that it follows from.
 fs_status ctx_fail(fs_ctx* c, fs_status code, const std::string& msg);
+// the context of the call that this thread runs (for ctx_give_back)
+struct CtxScope {
+    fs_ctx* outer;
+    explicit CtxScope(fs_ctx* c);
+    ~CtxScope();
+};
 template <typename Fn> fs_status ctx_call(fs_ctx* c, Fn fn) {
+    CtxScope scope(c);
     try {
         fn();
         ctx_check_errflag(c);
@@ -473,8 +500,9 @@ struct OzDst {
     long cm, cn;
     const int *mmap = nullptr, *nmap = nullptr;
 };
+// false: no memory for its images, nothing done
 bool oz_worth(int M, int N, int K);
-void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& A, const OzMat& B, const OzDst& C, double alpha, double beta,
+bool oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& A, const OzMat& B, const OzDst& C, double alpha, double beta,
              int table = 0);
 
 // dense FP64 linear algebra (fs_dense.cu); column-major complex, op 0 = N, 1 = C

@@ -880,10 +880,7 @@ void dense_gemm_mat(fs_ctx* c, int M, int N, int K, double alpha, const OzMat& A
                     const OzDst& C, int table, int lower) {
     if (M <= 0 || N <= 0) return;
     K = std::max(K, 0);
-    if (!lower && oz_worth(M, N, K)) {
-        oz_gemm(c, M, N, K, A, B, C, alpha, beta, table);
-        return;
-    }
+    if (!lower && oz_worth(M, N, K) && oz_gemm(c, M, N, K, A, B, C, alpha, beta, table)) return;
     const int tiles = cdiv(M, TB) * cdiv(N, TB);
     int splits = 1;
     if (tiles < 4 * 152) splits = std::min(std::max(1, 4 * 152 / tiles), std::max(1, K / (2 * TK)));

@@ -573,21 +573,32 @@ void fmt(fs_ctx* c, const OzOp& op, int r0, int R, int K, int rows, int tr, int 
 
 }  // namespace
 
-// sizes from which the tensor-core form is taken (see dense_gemm_impl)
+// sizes from which the tensor-core form is taken (see dense_gemm_mat)
 bool oz_worth(int M, int N, int K) { return 8.0 * M * N * (double)K >= 6e7 && K >= 64 && std::max(M, N) >= 32; }
+
+// Whether the context may keep a digit image of `bytes` of its projector table: small ones always,
+// others while they take at most an eighth of the memory then free, so that the library's and the
+// program's other buffers find the room they had.
+static bool image_fits(size_t bytes) {
+    if (bytes <= 256ull << 20) return true;
+    if (bytes > FS_TABLE_FMT_MAX_BYTES) return false;
+    size_t avail = 0, total = 0;
+    FS_CUDA(cudaMemGetInfo(&avail, &total));
+    return bytes <= avail / 8;
+}
 
 // C(m, n) = alpha sum_k a(m, k) b(k, n) + beta C(m, n) on the tensor cores (header of this file).
 // Of the two ways round (either operand as the 128-row side) the one with less padded work is taken.
-void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, const OzDst& Cd, double alpha,
+// Every buffer is allocated before the first launch; where the images do not fit, they are made in
+// smaller chunks, and false is returned if that does not help either.
+bool oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, const OzDst& Cd, double alpha,
              double beta, int table) {
     auto cost = [](int m, int n) {  // tiles x cycles of an MMA: shared-memory reads of both operands
         const int jt = cdiv_(n, ON2_MAX / 2), n2 = 2 * cdiv_(cdiv_(n, jt), 8) * 8;
         return (double)cdiv_(m, OM) * jt * (32 + n2 / 4);
     };
-    if (!table && cost(N, M) < cost(M, N)) {
-        oz_gemm(c, N, M, K, Bm, Am, OzDst{Cd.C, Cd.cn, Cd.cm, Cd.nmap, Cd.mmap}, alpha, beta, -1);
-        return;
-    }
+    if (!table && cost(N, M) < cost(M, N))
+        return oz_gemm(c, N, M, K, Bm, Am, OzDst{Cd.C, Cd.cn, Cd.cm, Cd.nmap, Cd.mmap}, alpha, beta, -1);
     table = std::max(table, 0);
     const int conja = Am.conj, conjb = Bm.conj;
     std::call_once(g_oz_attr, [] {
@@ -604,74 +615,85 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
     const size_t bstage = (size_t)NS * N2 * 32;
     dbuf* keep = table == 1 ? &W.table_g : table == 2 ? &W.table_n : nullptr;
     dbuf* keepm = table == 1 ? &W.max_g : &W.max_n;
+    bool* have = table == 1 ? &W.have_g : &W.have_n;
     const size_t abytes = (size_t)itiles * nkb * OA_STAGE;
-    if (keep && !keep->p && abytes > FS_TABLE_FMT_MAX_BYTES) keep = nullptr;
-    W.ma.ensure((size_t)M * sizeof(unsigned long long));
-    W.mb.ensure((size_t)N * sizeof(unsigned long long));
-    unsigned long long* ma = W.ma.as<unsigned long long>();
-    unsigned long long* mb = W.mb.as<unsigned long long>();
-    const size_t OZ_CHUNK_BYTES = 1ull << 30;
+    if (keep && !*have && (W.no_image || !image_fits(abytes) || !keepm->try_ensure((size_t)M * sizeof(unsigned long long)) ||
+                           !keep->try_ensure(abytes))) {
+        W.no_image = true;
+        keep = nullptr;
+    }
     // an operand is scaled and formatted in one launch (all of K at once) while that leaves a block
     // at most 16,384 elements (8 rows along k, 32 rows contiguous in memory) or there are blocks for
     // every SM; else maxima first, and by chunks of k.  (64 rows of 5,514 in eight blocks took 100 us
     // longer than three launches.)
     const bool onea = a.sk == 1 ? K <= 2048 || (K <= 8192 && M >= 8 * 152) : K <= 512 || M >= 32 * 152;
     const bool oneb = b.sk == 1 ? K <= 2048 || (K <= 8192 && N >= 8 * 152) : K <= 512 || N >= 32 * 152;
-    // stages per chunk and row tiles per chunk of the per-call images (at most OZ_CHUNK_BYTES each)
-    int kch = nkb, ich = itiles;
-    if (!keep) {
-        // long rows (Gram form): chunks of k; many rows (apply form): chunks of rows
-        if ((size_t)nkb * OA_STAGE * std::min(itiles, 16) > OZ_CHUNK_BYTES)
-            kch = (int)std::max<size_t>(64, OZ_CHUNK_BYTES / ((size_t)OA_STAGE * itiles));
-        else
-            ich = (int)std::max<size_t>(1, std::min<size_t>(itiles, OZ_CHUNK_BYTES / ((size_t)nkb * OA_STAGE)));
-    }
-    kch = (int)std::max<size_t>(64, std::min<size_t>(kch, OZ_CHUNK_BYTES / (bstage * jtiles)));
-    kch = std::min(nkb, cdiv_(kch, OCHAIN) * OCHAIN);
-    if (kch < nkb) ich = itiles;
-    const bool whole = kch == nkb;
-    if (keep) {
-        if (!keep->p) {
-            keepm->ensure((size_t)M * sizeof(unsigned long long));
-            keep->alloc(abytes);
-            unsigned long long* mx = keepm->as<unsigned long long>();
-            if (onea) {
-                maxfmt<false>(c, a, 0, M, K, itiles * OM, 0, nkb, 0, 0, mx, keep->as<unsigned char>());
-            } else {
-                row_max(c, a, M, K, mx);
-                fmt<false>(c, a, 0, M, K, itiles * OM, 0, 0, nkb, 0, 0, mx, keep->as<unsigned char>());
-            }
+    // stages per chunk and row tiles per chunk of the per-call images (at most `limit` bytes each)
+    int kch = nkb, ich = itiles, ztot = 0;
+    auto per_split = [&](int nk) {  // stages per split of a chunk over the grid's z: fill the SMs, whole chains
+        const int want = std::max(1, (N2 <= 16 ? 2 : 1) * 152 / (jtiles * std::min(ich, itiles)));
+        const int splits = std::max(1, std::min({want, nk / (2 * OCHAIN), 4096}));
+        return cdiv_(cdiv_(nk, splits), OCHAIN) * OCHAIN;
+    };
+    auto plan = [&](size_t limit) {
+        kch = nkb;
+        ich = itiles;
+        if (!keep) {
+            // long rows (Gram form): chunks of k; many rows (apply form): chunks of rows
+            if ((size_t)nkb * OA_STAGE * std::min(itiles, 16) > limit)
+                kch = (int)std::max<size_t>(64, limit / ((size_t)OA_STAGE * itiles));
+            else
+                ich = (int)std::max<size_t>(1, std::min<size_t>(itiles, limit / ((size_t)nkb * OA_STAGE)));
         }
+        kch = (int)std::max<size_t>(64, std::min<size_t>(kch, limit / (bstage * jtiles)));
+        kch = std::min(nkb, cdiv_(kch, OCHAIN) * OCHAIN);
+        if (kch < nkb) ich = itiles;
+        ztot = 0;
+        for (int k0 = 0; k0 < nkb; k0 += kch) {
+            const int nk = std::min(kch, nkb - k0);
+            ztot += cdiv_(nk, per_split(nk));
+        }
+        return W.mb.try_ensure((size_t)N * sizeof(unsigned long long)) &&
+               (keep || (W.ma.try_ensure((size_t)M * sizeof(unsigned long long)) &&
+                         W.aimg.try_ensure((size_t)ich * kch * OA_STAGE))) &&
+               W.bimg.try_ensure((size_t)jtiles * kch * bstage) &&
+               (ztot == 1 || W.part.try_ensure((size_t)ztot * M * N * sizeof(double2)));
+    };
+    bool fits = false;
+    for (size_t limit = 1ull << 30; !fits && limit >= 1ull << 24;) {
+        fits = plan(limit);
+        if (keep && !keep->p)  // given back for one of the buffers
+            keep = nullptr, fits = false;
+        else if (!fits)
+            limit >>= 3;
+    }
+    if (!fits) return false;
+    const bool whole = kch == nkb;
+    unsigned long long* ma = W.ma.as<unsigned long long>();
+    unsigned long long* mb = W.mb.as<unsigned long long>();
+    if (keep) {
         ma = keepm->as<unsigned long long>();
+        if (!*have) {
+            if (onea) {
+                maxfmt<false>(c, a, 0, M, K, itiles * OM, 0, nkb, 0, 0, ma, keep->as<unsigned char>());
+            } else {
+                row_max(c, a, M, K, ma);
+                fmt<false>(c, a, 0, M, K, itiles * OM, 0, 0, nkb, 0, 0, ma, keep->as<unsigned char>());
+            }
+            FS_CUDA(cudaGetLastError());
+            *have = true;
+        }
     } else if (!(onea && whole)) {
         row_max(c, a, M, K, ma);
     }
     if (!(oneb && whole)) row_max(c, b, N, K, mb);
-    // split of a chunk's stages over the grid's z: fill the SMs, whole chains per split
-    auto splits_of = [&](int nk) {
-        const int tiles = jtiles * std::min(ich, itiles);
-        const int want = std::max(1, (N2 <= 16 ? 2 : 1) * 152 / tiles);
-        return std::max(1, std::min({want, nk / (2 * OCHAIN), 4096}));
-    };
-    std::vector<int> zs;
-    int ztot = 0;
-    for (int k0 = 0; k0 < nkb; k0 += kch) {
-        const int nk = std::min(kch, nkb - k0), per = cdiv_(cdiv_(nk, splits_of(nk)), OCHAIN) * OCHAIN;
-        zs.push_back(per);
-        ztot += cdiv_(nk, per);
-    }
-    OzOut o{Cd.C, Cd.cm, Cd.cn, Cd.mmap, Cd.nmap, alpha, beta, nullptr};
-    if (ztot > 1) {
-        W.part.ensure((size_t)ztot * M * N * sizeof(double2));
-        o.part = W.part.as<double2>();
-    }
+    OzOut o{Cd.C, Cd.cm, Cd.cn, Cd.mmap, Cd.nmap, alpha, beta, ztot > 1 ? W.part.as<double2>() : nullptr};
     const size_t sbytes = OA_STAGE + bstage;
     const auto kernel = N2 <= 16 ? oz_gemm_kernel<1> : N2 <= 32 ? oz_gemm_kernel<2> : oz_gemm_kernel<4>;
     const int nst = (int)std::min<size_t>(O_STAGES_MAX, ((N2 <= 16 ? 112 * 1024 : O_SMEM_MAX) - O_CTL) / sbytes);
-    int z0 = 0, q = 0;
-    for (int k0 = 0; k0 < nkb; k0 += kch, ++q) {
-        const int nk = std::min(kch, nkb - k0), per = zs[q], nz = cdiv_(nk, per);
-        W.bimg.ensure((size_t)jtiles * nk * bstage);
+    int z0 = 0;
+    for (int k0 = 0; k0 < nkb; k0 += kch) {
+        const int nk = std::min(kch, nkb - k0), per = per_split(nk), nz = cdiv_(nk, per);
         if (oneb && whole)
             maxfmt<true>(c, b, 0, N, K, jtiles * tr, tr, nkb, conja, conjb, mb, W.bimg.as<unsigned char>());
         else
@@ -685,7 +707,6 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
                 stride = nkb;
                 akb = k0;
             } else {
-                W.aimg.ensure((size_t)ni * nk * OA_STAGE);
                 if (onea && whole)
                     maxfmt<false>(c, a, i0 * OM, M, K, ni * OM, 0, nkb, 0, 0, ma, W.aimg.as<unsigned char>());
                 else
@@ -707,4 +728,5 @@ void oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
     if (ztot > 1)
         oz_sum_kernel<<<cdiv_((long)M * N, 32), 256, 0, c->stream>>>(M, N, ztot, o);
     FS_CUDA(cudaGetLastError());
+    return true;
 }
