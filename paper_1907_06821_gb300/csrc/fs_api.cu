@@ -305,6 +305,7 @@ fs_status fs_create(const fs_grid* grid, double ecut, const double k[3], const d
             throw fs_error(FS_ERR_ARG, "bad gemm_path");
         c->gemm_path = c->opt.gemm_path;
         FS_CUDA(cudaGetDevice(&c->device));
+        FS_CUDA(cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device));
         c->errflag = flag_take();
         FS_CUDA(cudaHostGetDevicePointer((void**)&c->errflag_dev, c->errflag, 0));
         if (c->opt.cuda_stream) {

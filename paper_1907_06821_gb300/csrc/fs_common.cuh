@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <initializer_list>
 #include <new>
 #include <string>
 #include <vector>
@@ -288,6 +289,8 @@ struct fs_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int device = 0;   // the device that was current at fs_create (every buffer lives there)
+    int nsm = 0;      // its SMs
+    bool tc_limit = false, oz_limit = false, mlp_fwd_limit = false, mlp_grad_limit = false;  // smem_limit done
 
     // basis tables (device)
     dbuf col_start;   // int [ncol+1]
@@ -362,6 +365,16 @@ struct fs_ctx {
     int gemm_path = 0;
     std::string err;
 };
+
+// Dynamic shared-memory limit of kernels, raised once per context: the attribute belongs to the
+// kernel on one device (and to its context there), so a flag of the process would leave the
+// launches of a context on another device to fail.
+inline void smem_limit(bool& done, int bytes, std::initializer_list<const void*> kernels) {
+    if (done) return;
+    for (const void* k : kernels)
+        FS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    done = true;
+}
 
 void prof_flush(fs_ctx* c);
 void prof_release(fs_ctx* c);

@@ -17,7 +17,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 #include <random>
 
 namespace {
@@ -782,16 +781,8 @@ void mlp_prepare(fs_ctx* c) {
 void mlp_forward(fs_ctx* c, const float* F, int rows, float* z) {
     if (rows <= 0) return;
     ProfScope ps(c, KS_VECTOR, rows * 20.0, rows * 2.0 * (4 * H + 2 * H * H + H));
-    static bool attr = false;
-    if (!attr) {
-        FS_CUDA(cudaFuncSetAttribute((const void*)mlp_forward_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     TC_SMEM));
-        attr = true;
-    }
-    int dev = 0, nsm = 0;
-    FS_CUDA(cudaGetDevice(&dev));
-    FS_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int grid = std::max(1, std::min((rows + MT - 1) / MT, nsm));
+    smem_limit(c->mlp_fwd_limit, TC_SMEM, {(const void*)mlp_forward_tc_kernel});
+    const int grid = std::max(1, std::min((rows + MT - 1) / MT, c->nsm));
     mlp_forward_tc_kernel<<<grid, MT, TC_SMEM, c->stream>>>(c->mlp.P.as<float>(), c->mlp.T.as<float>(), F, rows, z,
                                                             ctx_errflag(c));
     FS_CUDA(cudaGetLastError());
@@ -812,14 +803,8 @@ double mlp_weight_sum(fs_ctx* c, const float* wt, int rows) {
 double mlp_loss_grad(fs_ctx* c, const float* F, const float* zt, const float* wt, int rows, double sw) {
     Mlp& L = c->mlp;
     if (rows <= 0) throw fs_error(FS_ERR_CUDA, "no training rows");
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute((const void*)mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
-    });
-    int dev = 0, nsm = 0;
-    FS_CUDA(cudaGetDevice(&dev));
-    FS_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int nblk = (int)std::max(1l, std::min(((long)rows + GR - 1) / GR, (long)nsm));
+    smem_limit(c->mlp_grad_limit, G_SMEM, {(const void*)mlp_grad_kernel});
+    const int nblk = (int)std::max(1l, std::min(((long)rows + GR - 1) / GR, (long)c->nsm));
     L.gpart.ensure((size_t)nblk * 2 * NPAD * sizeof(float));
     mlp_grad_kernel<<<nblk, GT, G_SMEM, c->stream>>>(L.P.as<float>(), F, zt, wt, rows, (float)(1.0 / sw),
                                                      L.gpart.as<float>());

@@ -40,7 +40,6 @@
 #include <algorithm>
 #include <cfloat>
 #include <climits>
-#include <mutex>
 
 namespace {
 
@@ -546,8 +545,6 @@ __global__ void __launch_bounds__(256) oz_sum_kernel(int M, int N, int splits, O
 
 inline int cdiv_(long a, long b) { return (int)((a + b - 1) / b); }
 
-std::once_flag g_oz_attr;
-
 void row_max(fs_ctx* c, const OzOp& op, int R, int K, unsigned long long* out) {
     FS_CUDA(cudaMemsetAsync(out, 0, (size_t)R * sizeof(unsigned long long), c->stream));
     const int bx = op.sk == 1 ? cdiv_(R, 8) : cdiv_(R, 256);
@@ -601,11 +598,8 @@ bool oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
         return oz_gemm(c, N, M, K, Bm, Am, OzDst{Cd.C, Cd.cn, Cd.cm, Cd.nmap, Cd.mmap}, alpha, beta, -1);
     table = std::max(table, 0);
     const int conja = Am.conj, conjb = Bm.conj;
-    std::call_once(g_oz_attr, [] {
-        for (const void* k : {(const void*)oz_gemm_kernel<1>, (const void*)oz_gemm_kernel<2>,
-                              (const void*)oz_gemm_kernel<4>})
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, O_SMEM_MAX);
-    });
+    smem_limit(c->oz_limit, O_SMEM_MAX,
+               {(const void*)oz_gemm_kernel<1>, (const void*)oz_gemm_kernel<2>, (const void*)oz_gemm_kernel<4>});
     OzWork& W = c->oz;
     const OzOp a{Am.X, Am.sr, Am.sk, Am.map, Am.kmap, Am.rp, Am.kp},
         b{Bm.X, Bm.sr, Bm.sk, Bm.map, Bm.kmap, Bm.rp, Bm.kp};

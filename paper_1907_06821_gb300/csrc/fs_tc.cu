@@ -40,7 +40,6 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
-#include <mutex>
 #include <type_traits>
 
 namespace {
@@ -672,17 +671,6 @@ __global__ void wait_selftest_kernel(long long limit, int* errflag) {
     }
 }
 
-std::once_flag g_attr_once;
-int g_nsm = 0;
-void set_attrs() {
-    std::call_once(g_attr_once, [] {
-        cudaFuncSetAttribute((const void*)tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX);
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&g_nsm, cudaDevAttrMultiProcessorCount, dev);
-    });
-}
-
 inline int cdiv_(long a, long b) { return (int)((a + b - 1) / b); }
 
 // row maxima over k in [0, K)
@@ -725,7 +713,7 @@ struct TcDst64 {
 template <class OpA, class OpB>
 void tc_run(fs_ctx* c, int M, int N, int K, const OpA& a, int acont, int amaxk, const OpB& b, int bcont, int conja,
             dbuf* keep, dbuf* keepm, const TcDst64* d64, TcOut o, int lower = 0) {
-    set_attrs();
+    smem_limit(c->tc_limit, TC_SMEM_MAX, {(const void*)tc_gemm_kernel});
     const int nkb = std::max(1, cdiv_(K, KC)), itiles = cdiv_(M, TM);
     const int jtiles = cdiv_(N, TN2_MAX / 2);
     const int tr = cdiv_(cdiv_(N, jtiles), 8) * 8, N2 = 2 * tr;  // columns of C per tile, balanced
@@ -781,9 +769,9 @@ void tc_run(fs_ctx* c, int M, int N, int K, const OpA& a, int acont, int amaxk, 
         int best = 1;
         if (d64) {
             double eff_best = 0;
-            const int most = std::max(1, std::min(nk / (2 * CHAIN), cdiv_(4 * g_nsm, tiles)));
+            const int most = std::max(1, std::min(nk / (2 * CHAIN), cdiv_(4 * c->nsm, tiles)));
             for (int sp = 1; sp <= most; ++sp) {
-                const double eff = (double)tiles * sp / ((double)cdiv_((long)tiles * sp, g_nsm) * g_nsm);
+                const double eff = (double)tiles * sp / ((double)cdiv_((long)tiles * sp, c->nsm) * c->nsm);
                 if (eff > eff_best + 1e-9) {
                     eff_best = eff;
                     best = sp;
@@ -829,7 +817,7 @@ void tc_run(fs_ctx* c, int M, int N, int K, const OpA& a, int acont, int amaxk, 
                 format_a(i0, ni, k0, nk, ma, c->afmt.as<unsigned char>());
                 Af = c->afmt.as<unsigned char>();
             }
-            const int ntiles = jtiles * ni * nz, grid = std::min(ntiles, g_nsm);
+            const int ntiles = jtiles * ni * nz, grid = std::min(ntiles, c->nsm);
             tc_gemm_kernel<<<grid, TC_THREADS, (size_t)nst * sbytes + TC_CTL, c->stream>>>(
                 M, N, i0 * TM, N2, ni, jtiles, ntiles, nk, per, nst, lower, Af, stride, akb, c->bfmt.as<unsigned char>(), ma,
                 mb, o, z0, ctx_errflag(c));
