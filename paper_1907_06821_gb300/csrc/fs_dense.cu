@@ -1044,7 +1044,7 @@ void dense_heev(fs_ctx* c, int n, double2* A, int m, double* w, double2* Z, int 
         D.attr_set = true;
     }
     // a block per column, at most one per SM; the columns in shared memory when they fit
-    // (n <= 1216 on 152 SMs)
+    // (n <= 1296 on 152 SMs)
     const int nblocks = std::max(1, std::min(nsm, n - 1));
     const size_t vecs = (size_t)2 * n * sizeof(double2) + (size_t)cdiv(n, nblocks) * (ht / 32) * sizeof(double2);
     const size_t own = (size_t)cdiv(n, nblocks) * n * sizeof(double2);

@@ -1,5 +1,7 @@
-"""Accuracy of the dense eigensolver where the way it computes shows: small matrices, and rows
-of very different size."""
+"""Accuracy of the dense eigensolver where the way it computes shows: small matrices, rows of very
+different size, close eigenvalues, the reduction in place, several reductions at once."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -89,3 +91,54 @@ def test_scaled_and_indefinite_b(ctx):
         with pytest.raises(FSError, match="column") as ei:
             ctx.dense_eigh(A, m=4, B=C)
         assert ei.value.code == FS_ERR_NUMERIC
+
+
+# the reduction keeps its columns in shared memory up to 1,296 rows on 152 SMs, else in place;
+# 2,048 is the largest size
+@pytest.mark.parametrize("n", [1296, 1297, 2048])
+def test_reduction_in_place(ctx, n):
+    A = _herm(np.random.default_rng(n), n)
+    w, Z = ctx.dense_eigh(A, m=7)
+    tol = 64 * n * U
+    assert np.abs(A @ Z - Z * w).max() < tol
+    assert np.abs(Z.conj().T @ Z - np.eye(7)).max() < tol
+
+
+# vectors of eigenvalues closer than 1e-13 of the norm are orthogonalised to one another in the
+# inverse iteration, the others by the Cholesky QR pass
+@pytest.mark.parametrize("gap", [1e-15, 5e-14, 2e-13, 1e-12, 1e-11, 1e-10])
+def test_close_eigenvalues(ctx, gap):
+    n, rng = 96, np.random.default_rng(17)
+    Q = np.linalg.qr(_herm(rng, n))[0]
+    lam = np.repeat(np.linspace(-1.0, 1.0, 12), 8) + gap * np.tile(np.arange(8), 12)
+    A = (Q * lam) @ Q.conj().T
+    A = (A + A.conj().T) / 2
+    w, Z = ctx.dense_eigh(A, m=n)
+    tol = 64 * n * U
+    assert np.abs(w - np.linalg.eigvalsh(A)).max() < tol
+    assert np.abs(A @ Z - Z * w).max() < tol
+    assert np.abs(Z.conj().T @ Z - np.eye(n)).max() < tol
+
+
+def test_several_reductions_at_once(fs):
+    """Three threads, each with a context and eigenproblems whose reduction takes more than half of
+    every SM's shared memory, so that two of them cannot be resident together: each runs to its end
+    (a cooperative launch starts when all of its blocks fit) and none gives up waiting."""
+    n, err = 1000, []
+    mats = [_herm(np.random.default_rng(s), n) for s in range(3)]
+    ref = [np.linalg.eigvalsh(A)[:8] for A in mats]
+
+    def work(i):
+        try:
+            with fs.Context((10.0, 10.0, 10.0), (16, 16, 16), 3.0, (0, 0, 0), np.zeros((16, 16, 16))) as c:
+                for _ in range(6):
+                    w, _ = c.dense_eigh(mats[i], m=8)
+                    assert np.abs(w - ref[i]).max() < 64 * n * U
+        except BaseException as e:  # noqa: BLE001 - reported by the main thread
+            err.append(e)
+    th = [threading.Thread(target=work, args=(i,)) for i in range(3)]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    assert not err, err
