@@ -188,7 +188,6 @@ fs_status fs_precond_loss_grad(fs_ctx* c, const float* features, const float* ta
         if (!(sw > 0)) throw fs_error(FS_ERR_ARG, "fs_precond_loss_grad: weights sum to zero");
         *loss = (float)mlp_loss_grad(c, features, target, weight, rows, sw);
         FS_CUDA(cudaMemcpyAsync(grad, c->mlp.g.p, mlp_nparam() * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
-        FS_CUDA(cudaStreamSynchronize(c->stream));
     });
 }
 
