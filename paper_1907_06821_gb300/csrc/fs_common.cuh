@@ -107,7 +107,8 @@ struct fs_error {
 
 // ------------------------------------------------------------------ device buffer
 // Memory that the running call's context holds only to be faster (the FP64 digit images of its
-// projector table) is given back when an allocation fails; true if there was any (fs_api.cu).
+// projector table and of its last products) is given back when an allocation fails; true if there
+// was any (fs_api.cu).
 bool ctx_give_back();
 
 struct dbuf {
@@ -251,13 +252,19 @@ struct OzWork {
     dbuf table_g, table_n, max_g, max_n, aimg, bimg, ma, mb, part;
     bool have_g = false, have_n = false;  // the table image is complete
     bool no_image = false;                // there was no room for one: products go by chunks
+    bool busy = false;                    // a product is being set up: its own buffers stay
     bool give_back() {
         const bool any = table_g.p || table_n.p;
         table_g.release();
         table_n.release();
         have_g = have_n = false;
         no_image = no_image || any;
-        return any;
+        if (busy) return any;
+        const bool more = aimg.p || bimg.p || part.p;
+        aimg.release();
+        bimg.release();
+        part.release();
+        return any || more;
     }
 };
 

@@ -601,6 +601,11 @@ bool oz_gemm(fs_ctx* c, int M, int N, int K, const OzMat& Am, const OzMat& Bm, c
     smem_limit(c->oz_limit, O_SMEM_MAX,
                {(const void*)oz_gemm_kernel<1>, (const void*)oz_gemm_kernel<2>, (const void*)oz_gemm_kernel<4>});
     OzWork& W = c->oz;
+    struct Busy {
+        bool& b;
+        explicit Busy(bool& x) : b(x) { b = true; }
+        ~Busy() { b = false; }
+    } busy(W.busy);
     const OzOp a{Am.X, Am.sr, Am.sk, Am.map, Am.kmap, Am.rp, Am.kp},
         b{Bm.X, Bm.sr, Bm.sk, Bm.map, Bm.kmap, Bm.rp, Bm.kp};
     const int nkb = cdiv_(K, OKC), itiles = cdiv_(M, OM);

@@ -78,3 +78,19 @@ def test_images_are_given_back(fs):
             assert c.chebfd(0.0, 0.3, -12.0, 13.0, 4, 256, 1)["nfound"] == want
             c.apply_H(x, out=out, shift=0.1)
         assert (out - ref).abs().max().item() < 1e-12 * ref.abs().max().item()
+
+
+def test_images_of_products_are_given_back(fs):
+    """The same for the images of an earlier call's operands (0.6 GB; projectors formed where they
+    are used have no table to keep an image of)."""
+    w = fi.make_medium()
+    with fs.Context.from_workload(w, precision=fs.FS_FP64, projectors=fs.FS_PROJ_GENERATED) as c:
+        want = c.chebfd(0.0, 0.3, -12.0, 13.0, 4, 160, 1)["nfound"]
+    with fs.Context.from_workload(w, precision=fs.FS_FP64, projectors=fs.FS_PROJ_GENERATED) as c:
+        x = _bands(c, 16, 3)
+        out = c.apply_H(x, shift=0.1)
+        ref = out.clone()
+        with Ballast(300 << 20):
+            assert c.chebfd(0.0, 0.3, -12.0, 13.0, 4, 160, 1)["nfound"] == want
+            c.apply_H(x, out=out, shift=0.1)
+        assert (out - ref).abs().max().item() < 1e-12 * ref.abs().max().item()
