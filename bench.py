@@ -342,27 +342,29 @@ def make_line(args, w, ctx, results, stats, nconv, tmax, t_e2e, e2e_states, cloc
     g = ctx.gvectors()
     ncol = len(np.unique(np.asarray(g)[:, 0] * 100003 + np.asarray(g)[:, 1]))
     hpsi_bands = stats["col_inverse_fft"]["bytes"] / ((ctx.npw + w.n[2] * ncol) * 8.0)
-    # roofline of the library's dominant GEMM / FFT / vector class in the FP32 stage (the FP64
-    # dense algebra is latency- and FP64-bound, and the FP64 classes are the final check; their
-    # shares are reported in kernel_time_share and dense_la_parts)
-    own = {k: v for k, v in stats.items()
-           if k not in ("dense_la", "nonlocal_D") and not k.endswith("_fp64") and v["ms"] > 0}
-    top = max(own, key=lambda k: own[k]["ms"])
+    # roofline of the library's dominant GEMM / FFT / vector class in the stage the solve runs in (the
+    # FP64 dense algebra is latency- and FP64-bound, and in a mixed solve the FP64 classes are the
+    # final check; their shares are reported in kernel_time_share and dense_la_parts)
     fp32 = args.precision == "mixed"
+    own = {k: v for k, v in stats.items()
+           if k not in ("dense_la", "nonlocal_D") and k.endswith("_fp64") != fp32 and v["ms"] > 0}
+    top = max(own, key=lambda k: own[k]["ms"])
     st = stats[top]
     sec = st["ms"] / 1e3
     gbs = st["bytes"] / sec / 1e9                      # algorithmic bytes per second
     tfs = st["flops"] / sec / 1e12                     # algorithmic flops per second
     avg_bytes = st["bytes"] / max(st["launches"], 1)   # algorithmic bytes per launch
     traffic = NCU_TRAFFIC_RATIO[top] * avg_bytes if top in NCU_TRAFFIC_RATIO else None
-    if top in ("gram", "rotate", "nonlocal_project", "nonlocal_add"):
+    if top.removesuffix("_fp64") in ("gram", "rotate", "nonlocal_project", "nonlocal_add"):
         if fp32:
             # tcgen05 kind::f16 with a two-part FP16 split
             cpeak, cbound = bf16, "tensor"
             csrc = f"{src} bf16_tflops; the FP16 split runs 3 MMAs per product"
         else:
-            cpeak, cbound = 152 * 128 * 2 * 2.07e9 / 1e12 / 64, "alu"
-            csrc = "FP64 CUDA-core peak 152 SMs x 64 FMA x 2 x 2.07 GHz / 64 (GB300 FP64 rate)"
+            # products of 6e7 flops and more: exact 8-bit digits on tcgen05 kind::f16; the smaller ones
+            # run on the FP64 units (1.26 TFLOP/s), so a solve of small blocks stays below this
+            cpeak, cbound = bf16 / 34, "tensor"
+            csrc = f"{src} bf16_tflops / 34 (digit products per FP64 product)"
         # the binding resource is the one the kernel runs closer to
         if tfs / cpeak >= gbs / hbm:
             roof = {"kernel": top, "bound": cbound, "achieved": tfs, "peak": cpeak, "unit": "TFLOP/s",
