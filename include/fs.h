@@ -95,7 +95,10 @@ typedef struct {
     void* cuda_stream;         /* cudaStream_t to run on (NULL: the library's own stream) */
     int verbose;               /* > 0: one line per iteration on stderr */
     int gemm_path;             /* FP32-stage GEMMs: FS_GEMM_TENSOR (default, tcgen05, FP16 x3 split)
-                                  or FS_GEMM_CUDA_CORES (FP32 FMA); FP64 work always uses FP64 FMA */
+                                  or FS_GEMM_CUDA_CORES (FP32 FMA).  Not FP64 work: its products of
+                                  6e7 flops and more run on the tensor cores as exact products of
+                                  8-bit digits, accurate to 2^-55 of (largest entry of a row) x
+                                  (largest of a column), the smaller ones as FP64 FMA */
     int projectors;            /* FS_PROJ_AUTO (0, default): the projector table beta[N_p][npw] is
                                   stored when its FP64 form takes at most 16 GB, else generated;
                                   FS_PROJ_STORED; FS_PROJ_GENERATED: beta is formed where it is used

@@ -242,7 +242,7 @@ constexpr size_t FS_FMT_CHUNK_BYTES = 4ull << 30;
 // Workspace of the dense FP64 linear algebra (fs_dense.cu), kept by the context.
 #define FS_DENSE_MAX_N 2048
 struct DenseWork {
-    dbuf V, tau, d, e, e2, Y, z, work, info3, info, T, U, wyG, wyT, wyW, wyW2, gpart, qrG, qrT, linv, xb, ds, equil;
+    dbuf V, tau, d, e, e2, Y, z, info3, info, T, U, wyT, wyW, wyW2, gpart, qrG, qrT, linv, xb, ds, equil;
     bool attr_set = false;
 };
 

@@ -51,7 +51,7 @@ __device__ __forceinline__ double2 zconj(double2 a) { return make_double2(a.x, -
 // four FMAs per k in two chains.  (32 x 32 tiles with multiply-add-add took 1.5 operations
 // per product and left the SMs uneven; the row-mapped 64 x 64 tiles of the subspace
 // products took 1.9 ms for 36 x 36 x 1,069 on two SMs.  A plain FP64 solve of 8 states in
-// 1,069 plane waves: 1,069 -> 80 ms; eigensolve of n = 816 with its Cholesky: 55 -> 43 ms.)
+// 1,069 plane waves: 1,027 -> 80 ms; eigensolve of n = 816 with its Cholesky: 55 -> 43 ms.)
 // Split K (gridDim.z > 1): block z takes k in [z kc, min(K, (z + 1) kc)) and
 // writes its partial sum to part[(z N + n) M + m].
 // lower = 1: tiles wholly above the diagonal (every row index below every column

@@ -1,4 +1,7 @@
-// Complex GEMMs of the solver on CUDA cores (FP64 or FP32 operands).
+// Complex GEMMs of the solver: FP64 operands go to dense_gemm_mat (fs_dense.cu: digit products on
+// the tensor cores or FP64 FMA tiles), FP32 ones to the tensor cores (fs_tc.cu) or, with
+// FS_GEMM_CUDA_CORES, to the kernels here, which also serve the FP64 forms that dense_gemm_mat does
+// not have (D apart from C) and the allocation-free H application.
 //
 //   gemm_gram : C(i, j) = alpha * sum_k conj(A[i][k]) B[j][k] + beta * C(i, j)
 //               the inner products of two row blocks over the long plane-wave
@@ -9,7 +12,6 @@
 //               a small coefficient matrix applied to a row block (basis
 //               rotations, projector application).
 #include "fs_common.cuh"
-
 
 #include <algorithm>
 
