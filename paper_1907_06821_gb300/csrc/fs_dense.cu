@@ -288,9 +288,9 @@ __global__ void equil_sym_kernel(double2* A, double2* B, int n, const double* s)
     A[t] = cscale(cscale(A[t], fr), fc);
     B[t] = cscale(cscale(B[t], fr), fc);
 }
-__global__ void equil_rows_kernel(double2* Z, int n, int m, const double* s) {
+__global__ void equil_rows_kernel(const double2* Z, int n, int m, const double* s, double2* out) {
     const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (t < (long)n * m) Z[t] = cscale(Z[t], s[n + t % n]);
+    if (t < (long)n * m) out[t] = cscale(Z[t], s[n + t % n]);
 }
 
 // ------------------------------------------------------------------ tridiagonal reduction
@@ -1138,15 +1138,20 @@ void dense_heev(fs_ctx* c, int n, double2* A, int m, double* w, double2* Z, int 
 
 // Generalised Hermitian problem GA x = lambda GB x (both n x n, ld n; GB positive
 // definite): the m lowest pairs; eigenvectors (GB-orthonormal) overwrite GA's
-// first m columns, eigenvalues to w.  GB is overwritten (the Cholesky factor of the scaled GB).
+// first m columns, eigenvalues to w.  GB is overwritten.
 // Returns the Cholesky info (0 = success).
 int dense_hegv(fs_ctx* c, int n, double2* GA, double2* GB, int m, double* w) {
     DenseWork& D = c->dense;
+    // scaled where a product of the triangular solves goes to the tensor cores (n >= 315);
+    // the FMA products do not need it, and its launches are 8 us of 300 to 2,000 there
+    const bool scaled = oz_worth(std::max(std::min(n, IB), n - IB), n, std::min(n, IB));
     D.equil.ensure((size_t)2 * n * sizeof(double));
     const double* s = D.equil.as<double>();
-    equil_scale_kernel<<<cdiv(n, 256), 256, 0, c->stream>>>(GB, n, D.equil.as<double>());
-    equil_sym_kernel<<<cdiv((long)n * n, 256), 256, 0, c->stream>>>(GA, GB, n, s);
-    FS_CUDA(cudaGetLastError());
+    if (scaled) {
+        equil_scale_kernel<<<cdiv(n, 256), 256, 0, c->stream>>>(GB, n, D.equil.as<double>());
+        equil_sym_kernel<<<cdiv((long)n * n, 256), 256, 0, c->stream>>>(GA, GB, n, s);
+        FS_CUDA(cudaGetLastError());
+    }
     int info = dense_potrf(c, n, GB, n, nullptr);
     if (info != 0) return info;
     D.T.ensure((size_t)n * n * sizeof(double2));
@@ -1158,9 +1163,11 @@ int dense_hegv(fs_ctx* c, int n, double2* GA, double2* GB, int m, double* w) {
     dense_trsm(c, 0, n, n, GB, n, T, n, false);        // L^-1 GA L^-H
     dense_heev(c, n, T, m, w, D.U.as<double2>(), n);
     dense_trsm(c, 1, n, m, GB, n, D.U.as<double2>(), n, true);  // x = L^-H y
-    equil_rows_kernel<<<cdiv((long)n * m, 256), 256, 0, c->stream>>>(D.U.as<double2>(), n, m, s);
+    if (scaled)
+        equil_rows_kernel<<<cdiv((long)n * m, 256), 256, 0, c->stream>>>(D.U.as<double2>(), n, m, s, GA);
+    else
+        FS_CUDA(cudaMemcpyAsync(GA, D.U.p, (size_t)n * m * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
     FS_CUDA(cudaGetLastError());
-    FS_CUDA(cudaMemcpyAsync(GA, D.U.p, (size_t)n * m * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
     return 0;
 }
 

@@ -52,9 +52,9 @@ def test_multiples_of_the_unit_matrix(ctx):
         assert np.abs(Z.conj().T @ Z - np.eye(n)).max() < 64 * n * U
 
 
-# n = 600 and 816 take the triangular solves' products to the tensor cores; D runs up, down or
-# mixed over six (1e-6 .. 1) or twelve decades (1e-6 .. 1e6)
-@pytest.mark.parametrize("n,lo,hi", [(600, -6, 6), (816, -6, 0)])
+# the triangular solves' products go to the tensor cores, and the matrices are scaled, from n = 315
+# on; D runs up, down or mixed over six (1e-6 .. 1) or twelve decades (1e-6 .. 1e6)
+@pytest.mark.parametrize("n,lo,hi", [(120, -6, 6), (314, -6, 6), (315, -6, 6), (600, -6, 6), (816, -6, 0)])
 @pytest.mark.parametrize("order", ["up", "down", "mixed"])
 def test_graded_b(ctx, n, lo, hi, order):
     """A = D A' D, B = D B' D: the eigenvalues are those of (A', B') and Y = D Z is B'-orthonormal.
